@@ -90,7 +90,9 @@ typedef struct n2v_tune {
                               warps per SM where block_threads divides that, else 16, capped by
                               shared memory.  The persistent kernel is compiled for 128, 96, 80
                               and 64 registers a thread; the resident warps per SM (<= 16, 20,
-                              24, more) select the budget.                                    */
+                              24, more) select the budget.  Launches that step through sampled
+                              blocks (graphs with samples, no hub cache, merge form or block
+                              tier) take 24 warps where this is 0.                            */
   int32_t thread_max_deg;  /* a step runs on one lane when deg(v) and deg(t) are <= this      */
   int32_t smem_specials;   /* per-warp shared-memory slots for the special positions of a step */
   int32_t hub_count;       /* vertices (largest degree first) with a hashed neighbour set     */
@@ -151,7 +153,9 @@ typedef struct n2v_graph_info {
  * weighted graphs (8 bytes per entry) and the hub neighbour caches (the GPU
  * counterparts of the FN-Cache neighbour cache, Section 3.4): hashed
  * neighbour sets (8 bytes per slot) and rank bitmaps (16 bytes per 64
- * vertices of the graph, per bitmap hub). */
+ * vertices of the graph, per bitmap hub), and last the samples of col: one
+ * entry of every eight, half a byte for each entry.  n2v_graph_load also takes
+ * an aux that lacks only the room for the samples; walks are slower then. */
 int n2v_graph_aux_bytes(int64_t n, int64_t nnz, int weighted, const n2v_tune* t, size_t* bytes);
 
 /* Validate a device-resident CSR graph and build its auxiliary structures in
@@ -413,7 +417,9 @@ int n2v_step_stats(uint64_t* out, int32_t n, int32_t reset);
 
 /* Number of SMs and the persistent grid the handle would launch: blocks of
  * 128 threads, as many per SM as the tuning's resident warps ask for (20 by
- * default) and shared memory holds. */
+ * default) and shared memory holds.  (A launch that steps through sampled
+ * blocks needs less shared memory and takes its own number of blocks: see
+ * n2v_tune.blocks_per_sm.) */
 int n2v_launch_shape(const n2v_graph* g, int32_t* sms, int32_t* blocks, int32_t* threads);
 
 #ifdef __cplusplus

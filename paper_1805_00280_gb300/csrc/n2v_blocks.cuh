@@ -1,0 +1,724 @@
+// The step through sampled blocks: membership in the longer list by a search of
+// its samples and one 32-byte block.
+//
+// col is read in blocks of eight entries (32 bytes: one DRAM sector), and the
+// auxiliary buffer keeps the first entry of every block, samples[i] = col[8 i]
+// (built by n2v_graph_load; half a byte for each entry of col).  The block that
+// can hold x is found among a row's samples, an eighth of the row, and whether it
+// holds x takes eight compares.  So a step reads the shorter list, the samples
+// beside its keys, and only those blocks of the longer list that a key falls
+// into: neighbouring keys share a block when the lists are of like length, and
+// when they are not most blocks are never read.
+//
+// Measured (GB300, R-MAT 24, p = 2, q = 0.5): staging the whole longer list read
+// 55 KB of lists a step; the blocks read 24 KB from DRAM and run 262,144-walk
+// launches in 83 ms against 134 ms.  Hashed sets of every row (one 32-byte bucket
+// a key, an eighth of the instructions) were built and measured as well: DRAM gives
+// 64 bytes for each random 32, 71 KB a step, and the same launches took 155 ms.
+//
+// A row starts and ends inside a block as a rule.  Entries of the neighbouring
+// rows there are told apart by their index, in the row's first and last block
+// only.
+#pragma once
+
+#include <type_traits>
+
+#include "n2v_step.cuh"
+
+namespace n2v {
+
+// A row as its blocks: block i holds the row's positions [8 i - head, 8 i + 8 - head).
+struct BlockRow {
+  const int32_t* __restrict__ smp;  // smp[i]: first entry of block i + 1, i < n1
+  const int32_t* __restrict__ blk;  // block i at blk + 8 i
+  int n1;    // samples inside the row (its blocks are 0 .. n1)
+  int head;  // entries of block 0 before the row
+  int len;
+  int cut;                           // the block that reaches past the end of col, or -1
+  const int32_t* __restrict__ tail;  // its copy
+};
+
+__device__ __forceinline__ BlockRow block_row(const GraphView& g, int64_t b, int d) {
+  BlockRow r;
+  const int64_t f = b >> 3;
+  r.smp = g.samples + f + 1;
+  r.blk = g.col + 8 * f;
+  r.n1 = (int)(((b + d - 1) >> 3) - f);
+  r.head = (int)(b & 7);
+  r.len = d;
+  r.cut = 8 * (f + r.n1 + 1) > g.nnz ? r.n1 : -1;
+  r.tail = g.samples + ((g.nnz + 31) >> 5 << 2);
+  return r;
+}
+
+struct Block {
+  int32_t s[8];
+};
+
+__device__ __forceinline__ Block block_at(const int32_t* p) {
+  const int4 x = __ldg((const int4*)p), y = __ldg((const int4*)p + 1);
+  return Block{{x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w}};
+}
+// Block i of the row (0 <= i <= n1).
+__device__ __forceinline__ Block block_load(const BlockRow& r, int i) {
+  return block_at(i == r.cut ? r.tail : r.blk + 8ll * i);
+}
+
+// Drop the entries of block i that belong to other rows (only the row's first and
+// last blocks have some).
+__device__ __forceinline__ void block_trim(const BlockRow& r, int i, Block& b) {
+  const unsigned at = (unsigned)(8 * i - r.head);
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (at + j >= (unsigned)r.len) b.s[j] = -1;
+}
+
+__device__ __forceinline__ bool block_has(const Block& b, int32_t x) {
+  return b.s[0] == x || b.s[1] == x || b.s[2] == x || b.s[3] == x || b.s[4] == x || b.s[5] == x || b.s[6] == x ||
+         b.s[7] == x;
+}
+
+// Position in the row of an x that the (trimmed) block i holds.
+__device__ __forceinline__ int block_pos(const BlockRow& r, int i, const Block& b, int32_t x) {
+  int p = 7;
+#pragma unroll
+  for (int j = 6; j >= 0; --j) p = b.s[j] == x ? j : p;
+  return 8 * i - r.head + p;
+}
+
+// First position of the row whose entry is >= x, given the block of x (the number
+// of samples <= x).
+__device__ __forceinline__ int block_lower_bound(const BlockRow& r, int i, const int32_t* __restrict__ row, int32_t x) {
+  const int lo = max(0, 8 * i - r.head), hi = min(r.len, 8 * i + 8 - r.head);
+  return lo + lower_bound32(row + lo, hi - lo, x);
+}
+
+// Blocks of N keys of one lane: the number of samples in [from, n1) at or below
+// each, plus from (N searches side by side).
+template <int N>
+__device__ __forceinline__ void block_search(const BlockRow& r, int from, const int32_t (&x)[N], int (&node)[N]) {
+#pragma unroll
+  for (int e = 0; e < N; ++e) node[e] = from;
+  const int n = r.n1 - from;
+  if (n <= 0) return;
+  for (int st = 1 << (31 - __clz(n)); st > 0; st >>= 1) {
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const int at = node[e] + st;
+      if (at <= r.n1 && __ldg(r.smp + at - 1) <= x[e]) node[e] = at;
+    }
+  }
+}
+
+// Parameters of a job that the steps share.
+struct StepArgs {
+  uint32_t a_p, a_q;
+  uint64_t inv_q;  // floor((2^64 - 1) / a_q)
+  uint64_t seed;
+};
+
+__device__ __forceinline__ uint64_t div_by_aq(const StepArgs& A, uint64_t x) {
+  uint64_t q = __umul64hi(x, A.inv_q);
+  if (x - q * (uint64_t)A.a_q >= (uint64_t)A.a_q) ++q;  // the estimate is the quotient or one less
+  return q;
+}
+
+// ---------------------------------------------------------------------------
+// One lane, one step (k >= 1), 1 <= deg v <= kLaneDeg: each neighbour of v is
+// looked up in N(t), four at a time, and the hits are kept as a bit mask.
+// Thirty-two walkers of a warp go side by side, so a step of 20 neighbours costs
+// a warp about 20 look-ups for 32 steps, where the warp-wide form below pays its
+// fixed cost once for each.
+constexpr int kLaneDeg = 64;
+
+template <bool W>
+__device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t bv, int dv, int64_t bt, int dt,
+                                                   int32_t t, uint64_t u, const StepArgs& A) {
+  const int32_t* __restrict__ nv = g.col + bv;
+  const uint64_t d1 = (uint64_t)kAlphaOne - (uint64_t)A.a_q, d2 = (uint64_t)A.a_p - (uint64_t)A.a_q;
+  uint64_t hits = 0;
+  int pt = kLaneDeg;  // index of t in N(v)
+  if (dt > 0) {
+    const BlockRow rt = block_row(g, bt, dt);
+    for (int i0 = 0; i0 < dv; i0 += 4) {
+      int32_t x[4];
+      int node[4];
+      Block b[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = __ldg(nv + min(i0 + e, dv - 1));
+      block_search<4>(rt, 0, x, node);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) b[e] = block_load(rt, node[e]);
+      uint32_t m = 0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        block_trim(rt, node[e], b[e]);
+        m |= block_has(b[e], x[e]) ? 1u << e : 0u;
+        if (x[e] == t) pt = min(pt, i0 + e);
+      }
+      hits |= (uint64_t)m << i0;
+    }
+    hits &= ~0ull >> (64 - dv);  // the last key, repeated past the end, sets no bit of its own
+  } else {
+    for (int i = 0; i < dv; ++i)
+      if (__ldg(nv + i) == t) pt = i;
+  }
+  if (pt < kLaneDeg) hits &= ~(1ull << pt);  // t weighs 1/p whatever N(t) holds
+  if (!W) {
+    const uint64_t T = (uint64_t)A.a_q * (uint64_t)dv + d1 * (uint64_t)__popcll(hits) + (pt < kLaneDeg ? d2 : 0ull);
+    const uint64_t r = scale_draw(u, T);
+    int lo = 0, n = dv - 1;  // the last position has C = T > r
+    while (n > 0) {
+      const int half = n >> 1, j = lo + half;
+      const uint64_t C = (uint64_t)A.a_q * (uint64_t)(j + 1) + d1 * (uint64_t)__popcll(hits & (~0ull >> (63 - j))) +
+                         (pt <= j ? d2 : 0ull);
+      if (C <= r) {
+        lo = j + 1;
+        n -= half + 1;
+      } else {
+        n = half;
+      }
+    }
+    return __ldg(nv + lo);
+  }
+  uint64_t T = (uint64_t)A.a_q * __ldg(g.wpre + bv + dv - 1);
+  for (uint64_t m = hits; m; m &= m - 1) T += d1 * (uint64_t)__ldg(g.w + bv + (__ffsll((long long)m) - 1));
+  if (pt < kLaneDeg) T += d2 * (uint64_t)__ldg(g.w + bv + pt);
+  if (T == 0) return -1;
+  const uint64_t r = scale_draw(u, T);
+  uint64_t C = 0;
+  int j = 0;
+  for (; j < dv - 1; ++j) {
+    const uint32_t a = j == pt ? A.a_p : ((hits >> j) & 1ull ? kAlphaOne : A.a_q);
+    C += (uint64_t)__ldg(g.w + bv + j) * a;
+    if (C > r) break;
+  }
+  return __ldg(nv + j);
+}
+
+// ---------------------------------------------------------------------------
+// Whole warp, one step (k >= 1, both degrees at least 1).  The keys are the
+// shorter list, in chunks of 32 and batches of four chunks.  The samples of the
+// longer list that lie between a batch's first and last key are staged in shared
+// memory (kWin at most; they follow on from the batch before, so each sample is
+// read once), every key finds its block there by a fixed-depth search, and the
+// batch's 128 blocks are loaded together.  Keys of a batch that spans more
+// samples search them in global memory.
+//
+// As in warp_step, C_j = a_q W_j + D_j, and T = a_q W_last + D_last needs only
+// how many keys hit (or the weights they hit).  What is kept of a chunk is its
+// ballot of hits and the block of its first key (with weights, also the sum over
+// its hits), not a list of positions.  When the chunks are more than the records,
+// one record keeps the total of a group of chunks, and the group that holds the
+// answer is gone through once more.
+//
+//   keys N(v), blocks of N(t): a key's index is its position, so C at the end of
+//     every chunk is known and the answer's chunk, then its lane, is found by
+//     ballots;
+//   keys N(t), blocks of N(v): a hit's position in N(v) is its lower bound there.
+//     It is taken for the first key of each chunk (one lane each, inside the
+//     recorded block), then for the 32 keys of the answer's chunk only.
+//
+// t itself (weight 1/p) is never counted as a hit: its part of D is added where
+// a position is at or behind it.
+constexpr int kWin = 512;         // staged samples per warp
+constexpr int32_t kNoKey = -2;    // in the place of a key past the end: below every vertex, equal to none
+
+// Shared memory of one warp: cap record words, cap more (the blocks of the first
+// keys; with weights the records take both), kWin samples.
+__host__ __device__ __forceinline__ int block_records(const LaunchCfg& L) {
+  return L.smem_specials < 1024 ? L.smem_specials : 1024;
+}
+__host__ __device__ __forceinline__ int block_smem_words(const LaunchCfg& L) { return 2 * block_records(L) + kWin; }
+
+template <bool W>
+struct BlockStep {
+  using Sum = typename std::conditional<W, uint64_t, uint32_t>::type;  // of hits, or of their weights
+  const GraphView& g;
+  const StepArgs& A;
+  const int64_t bv, bt;
+  const int dv, dt;
+  const int32_t t;
+  const int lane;
+  uint32_t* rec;
+  const int cap;
+  const int32_t* __restrict__ nv;
+  const int32_t* __restrict__ nt;
+
+  __device__ __forceinline__ int records() const { return W ? cap >> 1 : cap; }
+  // record i: total, ballot and first key's block
+  __device__ __forceinline__ void put_total(int i, Sum s) {
+    if (W) *(uint64_t*)(rec + 4 * i) = s;
+    else rec[i] = (uint32_t)s;
+  }
+  __device__ __forceinline__ Sum total_at(int i, int group) const {
+    if (W) return (Sum) * (const uint64_t*)(rec + 4 * i);
+    return group == 1 ? (Sum)__popc(rec[i]) : (Sum)rec[i];
+  }
+  __device__ __forceinline__ uint32_t ballot_at(int i) const { return W ? rec[4 * i + 2] : rec[i]; }
+  __device__ __forceinline__ uint32_t& block_of(int i) { return W ? rec[4 * i + 3] : rec[cap + i]; }
+
+  // static prefix of the positions before p
+  __device__ __forceinline__ uint64_t w_before(int p) const {
+    return W ? (p > 0 ? __ldg(g.wpre + bv + p - 1) : 0ull) : (uint64_t)p;
+  }
+  // first position in [lo, hi) of N(v) with an entry >= x (hi if none)
+  __device__ __forceinline__ int pos_of(int lo, int hi, int32_t x) const { return lo + lower_bound32(nv + lo, hi - lo, x); }
+
+  // The search of one staged level: p points at the first staged sample not yet known to
+  // be at or below the key.
+  template <int ST>
+  __device__ __forceinline__ static void level(uint32_t (&p)[4], const int32_t (&x)[4]) {
+    int32_t s[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) asm volatile("ld.shared.s32 %0, [%1+%2];" : "=r"(s[e]) : "r"(p[e]), "n"(4 * (ST - 1)));
+#pragma unroll
+    for (int e = 0; e < 4; ++e) p[e] += s[e] <= x[e] ? 4u * ST : 0u;
+  }
+
+  // State of a pass over the keys.
+  struct Pass {
+    const int32_t* __restrict__ keys;  // this lane's key of chunk 0
+    int nk;
+    int32_t kmax;          // the last key
+    int stage;             // samples staged for a batch at first: 64 or 128; 0: searched in global memory
+    int from;              // samples at or below every key still to come
+    int group;             // chunks that share one record (1, or a multiple of four)
+    int left, gi;          // of the current group: chunks to come, and its record
+    int32_t nx[4], ns[4];  // the next batch's keys and samples
+    Sum sum, before;       // hits so far, and before the group (with weights: this lane's share of their weights)
+    int pt;                // index of the key equal to t that this lane saw, or -1
+  };
+
+  __device__ __forceinline__ void fetch(Pass& P, const BlockRow& r, int c) const {
+    const int32_t* k = P.keys + 32 * c;
+    const int n = P.nk - 32 * c;
+    if (n >= 128) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) P.nx[e] = __ldg(k + 32 * e);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) P.nx[e] = 32 * e < n - lane ? __ldg(k + 32 * e) : kNoKey;
+    }
+    const int32_t* q = r.smp + P.from + lane;
+    const int m = r.n1 - P.from - lane;
+    P.ns[0] = 0 < m ? __ldg(q) : INT32_MAX;
+    P.ns[1] = 32 < m ? __ldg(q + 32) : INT32_MAX;
+    if (P.stage > 64) {
+      P.ns[2] = 64 < m ? __ldg(q + 64) : INT32_MAX;
+      P.ns[3] = 96 < m ? __ldg(q + 96) : INT32_MAX;
+    }
+  }
+
+  // One batch: chunks c .. c + 3.
+  __device__ __forceinline__ void batch(Pass& P, const BlockRow& r, int c, bool vk) {
+    int32_t* win = (int32_t*)(rec + 2 * cap);
+    int32_t x[4];
+    int node[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) x[e] = P.nx[e];
+    // the batch's largest key
+    const int32_t last = P.nk - 32 * c >= 128 ? __shfl_sync(kFull, x[3], 31) : P.kmax;
+    bool edges = P.from == 0;
+    int below = kWin;  // staged samples at or below the last key
+    if (P.stage) {
+      win[lane] = P.ns[0];
+      win[32 + lane] = P.ns[1];
+      below = (P.ns[0] <= last ? 1 : 0) + (P.ns[1] <= last ? 1 : 0);
+      if (P.stage > 64) {
+        win[64 + lane] = P.ns[2];
+        win[96 + lane] = P.ns[3];
+        below += (P.ns[2] <= last ? 1 : 0) + (P.ns[3] <= last ? 1 : 0);
+      }
+      below = __reduce_add_sync(kFull, below);
+      if (below == P.stage) {
+        int more = 0;
+#pragma unroll 2
+        for (int q = P.stage; q < kWin; q += 32) {
+          const int i = P.from + q + lane;
+          const int32_t s = i < r.n1 ? __ldg(r.smp + i) : INT32_MAX;
+          win[q + lane] = s;
+          more += s <= last ? 1 : 0;
+        }
+        below += __reduce_add_sync(kFull, more);
+      }
+      __syncwarp();
+    }
+    if (below < kWin) {
+      // samples at or below each key, by a search of 2^d - 1 >= below staged samples (the ones
+      // past `below` are above every key)
+      const uint32_t w0 = smem_addr(win);
+      uint32_t p[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) p[e] = w0;
+      if (below >= 32) {
+        if (below >= 128) {
+          if (below >= 256) level<256>(p, x);
+          level<128>(p, x);
+        }
+        if (below >= 64) level<64>(p, x);
+        level<32>(p, x);
+      }
+      if (below >= 8) {
+        if (below >= 16) level<16>(p, x);
+        level<8>(p, x);
+      }
+      level<4>(p, x);
+      level<2>(p, x);
+      level<1>(p, x);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) node[e] = P.from + (int)((p[e] - w0) >> 2);
+      P.from += below;
+    } else {
+      block_search<4>(r, P.from, x, node);
+      if (P.nk - 32 * c >= 128) P.from = __shfl_sync(kFull, node[3], 31);
+      else edges = true;  // the last batch
+    }
+    edges = edges || P.from == r.n1;
+    Block b[4];
+    if (r.cut < 0) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) b[e] = block_at(r.blk + 8ll * node[e]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) b[e] = block_load(r, node[e]);
+    }
+    if (32 * (c + 4) < P.nk) fetch(P, r, c + 4);
+    if (x[0] == t || x[1] == t || x[2] == t || x[3] == t) {  // t is no hit
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (x[e] == t) {
+          P.pt = 32 * (c + e) + lane;
+          x[e] = kNoKey;
+        }
+      }
+    }
+    if (edges) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) block_trim(r, node[e], b[e]);
+    }
+    uint32_t word[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool in = block_has(b[e], x[e]);
+      word[e] = __ballot_sync(kFull, in);
+      if (!W) {
+        P.sum += __popc(word[e]);
+      } else {
+        const int at = vk ? 32 * (c + e) + lane : block_pos(r, node[e], b[e], x[e]);
+        const uint32_t wx = in ? __ldg(g.w + bv + at) : 0u;
+        P.sum += wx;
+        if (P.group == 1) {  // this chunk's weights, in two halves that cannot overflow
+          const uint64_t cs = (uint64_t)__reduce_add_sync(kFull, wx & 0xffffu) +
+                              ((uint64_t)__reduce_add_sync(kFull, wx >> 16) << 16);
+          if (lane == 0) {
+            put_total(P.gi + e, (Sum)cs);
+            rec[4 * (P.gi + e) + 2] = word[e];
+            block_of(P.gi + e) = (uint32_t)node[e];
+          }
+        }
+      }
+    }
+    if (P.group == 1) {
+      if (!W && lane == 0) {
+        *(uint4*)(rec + P.gi) = make_uint4(word[0], word[1], word[2], word[3]);
+        *(uint4*)(rec + cap + P.gi) =
+            make_uint4((uint32_t)node[0], (uint32_t)node[1], (uint32_t)node[2], (uint32_t)node[3]);
+      }
+      P.gi += 4;
+    } else {
+      if (P.left == P.group && lane == 0) block_of(P.gi) = (uint32_t)node[0];
+      P.left -= 4;
+      if (P.left == 0 || 32 * (c + 4) >= P.nk) {
+        const Sum gs = W ? (Sum)warp_sum_u64(P.sum - P.before) : (Sum)(P.sum - P.before);
+        if (lane == 0) put_total(P.gi, gs);
+        P.before = P.sum;
+        P.left = P.group;
+        ++P.gi;
+      }
+    }
+    __syncwarp();  // the staged samples are read before the next batch's are written
+  }
+
+  // Look chunks [c0, c1) of the keys up in the longer list; the samples before `from`
+  // are at or below every key.  c1 - c0 is a multiple of four unless c1 ends the keys.
+  // Leaves a record for each group of chunks and returns the number of hits (with
+  // weights: this lane's share of their weights).
+  __device__ __forceinline__ Sum look_up(bool vk, const BlockRow& r, int from, int c0, int c1, int group, int* pt) {
+    Pass P;
+    P.keys = (vk ? nv : nt) + lane;
+    P.nk = vk ? dv : dt;
+    P.kmax = __ldg((vk ? nv : nt) + P.nk - 1);
+    // samples beside a batch of 128 keys: sixteen times the ratio of the lists
+    const int beside = r.len >> 3, nb = (P.nk + 127) >> 7;
+    P.stage = beside <= 48 * nb ? 64 : beside <= 400 * nb ? 128 : 0;
+    P.from = from;
+    P.group = group;
+    P.left = group;
+    P.gi = 0;
+    P.sum = 0;
+    P.before = 0;
+    P.pt = -1;
+    fetch(P, r, c0);
+#pragma unroll 1
+    for (int c = c0; c < c1; c += 4) batch(P, r, c, vk);
+    *pt = P.pt;
+    return P.sum;
+  }
+
+  // The same for at most 32 keys: one a lane, searched in global memory, one record.
+  __device__ __forceinline__ Sum look_up_one(bool vk, const BlockRow& r, int* pt) {
+    const int nk = vk ? dv : dt;
+    int32_t x[1] = {lane < nk ? __ldg((vk ? nv : nt) + lane) : kNoKey};
+    int node[1];
+    block_search<1>(r, 0, x, node);
+    Block b = block_load(r, node[0]);
+    block_trim(r, node[0], b);
+    *pt = x[0] == t ? lane : -1;
+    const bool in = block_has(b, x[0]) && x[0] != t;
+    const uint32_t word = __ballot_sync(kFull, in);
+    uint32_t wx = 0;
+    if (W && in) wx = __ldg(g.w + bv + (vk ? lane : block_pos(r, node[0], b, x[0])));
+    if (lane == 0) rec[W ? 2 : 0] = word;
+    __syncwarp();
+    return W ? (Sum)wx : (Sum)__popc(word);
+  }
+
+  // The chosen position in N(v), or -1 when T == 0.
+  __device__ __forceinline__ int run(uint64_t u) {
+    const uint64_t aq = A.a_q, d1 = (uint64_t)kAlphaOne - aq, d2 = (uint64_t)A.a_p - aq;
+    const bool vk = dv <= dt;
+    const int nk = vk ? dv : dt;
+    const BlockRow row = vk ? block_row(g, bt, dt) : block_row(g, bv, dv);
+    uint64_t t_part = 0;  // (1/p - 1/q) w(v, t) when t is in N(v)
+    int pos_t = -1;       // t's position in N(v), -1 when it is not there
+    if (!vk) {
+      pos_t = warp_find(t);
+      if (pos_t >= 0) t_part = d2 * (W ? (uint64_t)__ldg(g.w + bv + pos_t) : 1ull);
+    }
+    int c0 = 0, c1 = (nk + 31) >> 5;  // the chunks that can hold the answer
+    uint64_t D = 0;                   // the hits' part of D before chunk c0
+    int plo = 0, phi = dv;            // keys N(t): positions of the first keys of c0 and c1
+    uint64_t r = 0;
+    int from = 0;                     // samples at or below every key from c0 on
+    for (bool first = true;; first = false) {
+      const int nc = c1 - c0;
+      int group = 1;
+      if (nc > records()) group = ((nc + records() - 1) / records() + 3) & ~3;  // (a multiple of a batch)
+      const int n = (nc + group - 1) / group;
+      int pt = -1;
+      const Sum part = nk <= 32 ? look_up_one(vk, row, &pt) : look_up(vk, row, from, c0, c1, group, &pt);
+      if (first) {
+        if (vk) {
+          pos_t = __reduce_max_sync(kFull, pt);
+          if (pos_t >= 0) t_part = d2 * (W ? (uint64_t)__ldg(g.w + bv + pos_t) : 1ull);
+        }
+        const uint64_t all = W ? warp_sum_u64(part) : (uint64_t)part;
+        const uint64_t T = aq * w_before(dv) + d1 * all + t_part;
+        if (W && T == 0) return -1;
+        r = scale_draw(u, T);
+      }
+      // the record that holds the answer: the first whose end lies above r (keys N(v)), or the
+      // last whose first key's position has C at or below r just before it (keys N(t))
+      int pick = 0, npl = plo, nph = phi;
+      uint64_t Dp = D;
+      for (int i0 = 0; i0 < n && n > 1; i0 += 32) {
+        const int i = i0 + lane;
+        const Sum x = i < n ? total_at(i, group) : (Sum)0;
+        const Sum incl = W ? (Sum)warp_incl_scan_u64(x, lane) : (Sum)warp_incl_scan_u32((uint32_t)x, lane);
+        if (vk) {
+          const int pe = min(dv, 32 * (c0 + group * (i + 1)));
+          bool above = false;
+          if (i < n) above = aq * w_before(pe) + D + d1 * incl + (pos_t >= 0 && pos_t < pe ? t_part : 0ull) > r;
+          const unsigned m = __ballot_sync(kFull, above);
+          const Sum all = __shfl_sync(kFull, incl, 31);
+          if (m) {
+            const int f = __ffs(m) - 1;
+            pick = i0 + f;
+            Dp = D + d1 * __shfl_sync(kFull, (Sum)(incl - x), f);
+            break;
+          }
+          D += d1 * all;
+        } else {
+          int p = plo;
+          bool below = i == 0;
+          if (i > 0 && i < n) {
+            const int32_t y = __ldg(nt + 32 * (c0 + group * i));
+            p = block_lower_bound(row, (int)block_of(i), nv, y);
+            below = aq * w_before(p) + D + d1 * (Sum)(incl - x) + (pos_t >= 0 && pos_t < p ? t_part : 0ull) <= r;
+          }
+          const unsigned m = __ballot_sync(kFull, below);
+          const int f = 31 - __clz(m);  // -1: none of these
+          const Sum excl = __shfl_sync(kFull, (Sum)(incl - x), f & 31), all = __shfl_sync(kFull, incl, 31);
+          const int pf = __shfl_sync(kFull, p, f & 31), pn = __shfl_sync(kFull, p, (f + 1) & 31);
+          if (f >= 0) {
+            pick = i0 + f;
+            Dp = D + d1 * excl;
+            npl = pf;
+          }
+          if (f < 31) {  // the next record's first key bounds the answer
+            if (i0 + f + 1 < n) nph = pn;
+            break;
+          }
+          D += d1 * all;
+        }
+      }
+      D = Dp;
+      plo = npl;
+      phi = nph;
+      if (group == 1) {
+        const uint32_t word = ballot_at(pick);
+        return vk ? in_chunk_v(c0 + pick, word, D, pos_t, t_part, r)
+                  : in_chunk_t(c0 + pick, word, D, pos_t, t_part, plo, phi, r);
+      }
+      from = (int)block_of(pick);
+      c1 = min(c1, c0 + group * (pick + 1));
+      c0 += group * pick;
+      __syncwarp();  // every lane has read the records before they are written again
+    }
+  }
+
+  // Position of x in N(v), or -1: the warp narrows the list 32-fold with each load.
+  __device__ __forceinline__ int warp_find(int32_t x) const {
+    int lo = 0, n = dv;  // the first entry >= x is in [lo, lo + n]
+    while (n > 32) {
+      const int step = (n + 31) >> 5, i = lo + min((lane + 1) * step, n) - 1;
+      const unsigned m = __ballot_sync(kFull, __ldg(nv + i) < x);
+      const int f = __popc(m);  // the first f probes are below x
+      const int at = f * step;
+      if (at >= n) return -1;
+      lo += at;
+      n = min(step, n - at);
+    }
+    const unsigned m = __ballot_sync(kFull, lane < n && __ldg(nv + lo + lane) == x);
+    return m ? lo + __ffs(m) - 1 : -1;
+  }
+
+  // keys N(v): the answer lies in chunk c (hits: word), D before it
+  __device__ __forceinline__ int in_chunk_v(int c, uint32_t word, uint64_t D, int pos_t, uint64_t t_part, uint64_t r) {
+    const uint64_t d1 = (uint64_t)kAlphaOne - (uint64_t)A.a_q;
+    const int i = 32 * c + lane;
+    uint64_t own;
+    if (W) {
+      const uint64_t wx = ((word >> lane) & 1u) ? (uint64_t)__ldg(g.w + bv + i) : 0ull;
+      own = warp_incl_scan_u64(wx, lane);
+    } else {
+      own = (uint64_t)__popc(word & (0xffffffffu >> (31 - lane)));
+    }
+    bool above = false;
+    if (i < dv) above = (uint64_t)A.a_q * w_before(i + 1) + D + d1 * own + (pos_t >= 0 && pos_t <= i ? t_part : 0ull) > r;
+    const unsigned m = __ballot_sync(kFull, above);
+    N2V_CHECK(g, m != 0u);
+    return 32 * c + (m ? __ffs(m) - 1 : 0);
+  }
+
+  // keys N(t): the answer lies in [plo, phi), from the first key of chunk c on (hits: word)
+  __device__ __forceinline__ int in_chunk_t(int c, uint32_t word, uint64_t D, int pos_t, uint64_t t_part, int plo,
+                                            int phi, uint64_t r) {
+    const uint64_t aq = A.a_q, d1 = (uint64_t)kAlphaOne - aq;
+    const bool hit = (word >> lane) & 1u;
+    const int32_t y = hit ? __ldg(nt + 32 * c + lane) : 0;
+    const int p = hit ? pos_of(plo, phi, y) : 0;
+    uint64_t incl, own = hit ? 1ull : 0ull;
+    if (W) {
+      own = hit ? (uint64_t)__ldg(g.w + bv + p) : 0ull;
+      incl = warp_incl_scan_u64(own, lane);
+    } else {
+      incl = (uint64_t)__popc(word & (0xffffffffu >> (31 - lane)));
+    }
+    const bool below =
+        hit && aq * w_before(p) + D + d1 * (incl - own) + (pos_t >= 0 && pos_t < p ? t_part : 0ull) <= r;
+    const unsigned m = __ballot_sync(kFull, below);
+    int prev = plo - 1;  // the answer lies behind prev
+    if (m) {
+      const int f = 31 - __clz(m);
+      prev = __shfl_sync(kFull, p, f);
+      D += d1 * __shfl_sync(kFull, incl, f);
+      // the hit itself
+      if (aq * w_before(prev + 1) + D + (pos_t >= 0 && pos_t < prev ? t_part : 0ull) > r) return prev;
+    }
+    // behind prev every weight is the default up to the next hit, but for t
+    const bool passed = pos_t >= 0 && pos_t <= prev;
+    if (passed) D += t_part;
+    int j = first_above(prev, r - D);
+    if (pos_t >= 0 && !passed && j >= pos_t) {  // t lies in (prev, j]: nothing before it is above r
+      if (aq * w_before(pos_t + 1) + D + t_part > r) return pos_t;
+      j = first_above(pos_t, r - D - t_part);
+    }
+    N2V_CHECK(g, j >= plo && j < dv);
+    return j;
+  }
+
+  // First position behind prev whose a_q W exceeds x (the last one if none does).
+  __device__ __forceinline__ int first_above(int prev, uint64_t x) const {
+    const uint64_t m = div_by_aq(A, x);
+    if (W) return (int)warp_first_above_u64(g.wpre + bv, prev + 1, dv - 1, m, lane);
+    const int j = m > (uint64_t)(dv - 1) ? dv - 1 : (int)m;
+    return min(dv - 1, max(j, prev + 1));
+  }
+};
+
+// ---------------------------------------------------------------------------
+// One step of up to 32 walkers, one per lane.  On its lane: the first step, an
+// approximated step and the steps that are short enough; the others one after
+// another by the whole warp.
+template <bool W>
+__device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, int64_t t, int64_t v, int k, uint64_t wid,
+                                               const WalkJob& J, const StepArgs& A, int thr, uint32_t* rec, int cap,
+                                               int lane) {
+  enum { kDone, kLane, kMid, kWarp };
+  int how = kDone;
+  int32_t x = -1;
+  uint64_t u = 0;
+  int64_t bv = 0, bt = 0;
+  int dv = 0, dt = 0;
+  if (alive) {
+    bv = g.rp[v];
+    dv = (int)(g.rp[v + 1] - bv);
+    if (k > 0) {
+      bt = g.rp[t];
+      dt = (int)(g.rp[t + 1] - bt);
+    }
+    u = philox_draw(A.seed, wid, (uint32_t)k);
+    if (dv == 0) {
+      // a dead end
+    } else if (k == 0 || approx_here(J, k, dv, dt)) {
+      x = static_step(g, bv, bv + dv, u);
+    } else if (dv <= min(thr, kLaneDeg)) {
+      how = kLane;
+    } else {
+      how = thr > 0 && dv <= kLaneDeg ? kMid : kWarp;
+    }
+  }
+  // steps of up to kLaneDeg neighbours stay on their lanes when enough lanes have one
+  const bool together = __popc(__ballot_sync(kFull, how == kMid)) >= 8;
+  if (how == kLane || (together && how == kMid)) {
+    x = lane_block_step<W>(g, bv, dv, bt, dt, (int32_t)t, u, A);
+    how = kDone;
+  }
+  __syncwarp();
+  unsigned wm = __ballot_sync(kFull, how != kDone);
+  while (wm) {
+    const int src = __ffs(wm) - 1;
+    wm &= wm - 1;
+    const int64_t bv_ = __shfl_sync(kFull, bv, src), bt_ = __shfl_sync(kFull, bt, src);
+    BlockStep<W> st{g,
+                    A,
+                    bv_,
+                    bt_,
+                    __shfl_sync(kFull, dv, src),
+                    __shfl_sync(kFull, dt, src),
+                    __shfl_sync(kFull, (int32_t)t, src),
+                    lane,
+                    rec,
+                    cap,
+                    g.col + bv_,
+                    g.col + bt_};
+    const int j = st.run(__shfl_sync(kFull, u, src));
+    if (lane == src) x = j < 0 ? -1 : __ldg(g.col + bv + j);
+    __syncwarp();
+  }
+  return x;
+}
+
+}  // namespace n2v

@@ -55,6 +55,8 @@ AuxLayout aux_layout(int64_t n, int64_t nnz, int weighted, const n2v_tune& t) {
   L.bm_data = off;
   if (L.bm_cap > 0)
     off += align256(std::max<size_t>(16 * (size_t)L.bm_cap * (size_t)L.bm_words, 4 * ((size_t)n + 2)));
+  L.samples = off;  // one entry of every eight in col
+  off += align256(sizeof(int32_t) * (size_t)(((nnz + 31) >> 5 << 2) + 8));
   L.total = off;
   return L;
 }
@@ -290,6 +292,32 @@ static int build_bitmaps(n2v_graph* g, const AuxLayout& L, cudaStream_t s) {
   return N2V_OK;
 }
 
+// samples[i] = col[8 i]: the first entry of every 32-byte block of col.
+// Behind them goes a copy of the block that the end of col cuts, so that every block
+// can be loaded whole.
+__global__ void __launch_bounds__(256) k_samples(const int32_t* __restrict__ col, int64_t nnz,
+                                                 int32_t* __restrict__ samples) {
+  const int64_t blocks = (nnz + 7) >> 3;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < blocks; i += (int64_t)gridDim.x * blockDim.x)
+    samples[i] = __ldg(col + 8 * i);
+  if (blockIdx.x == 0 && threadIdx.x < 8) {
+    const int64_t e = (nnz & ~7ll) + threadIdx.x;
+    samples[((nnz + 31) >> 5 << 2) + threadIdx.x] = e < nnz ? __ldg(col + e) : -1;
+  }
+}
+
+// Take the samples of col into their part of aux (asynchronous).  A smaller aux,
+// enough for everything else, leaves them out: such a graph steps without them.
+static int build_samples(n2v_graph* g, const AuxLayout& L, cudaStream_t s) {
+  g->view.samples = nullptr;
+  if (g->nnz == 0 || g->aux_bytes < L.total) return N2V_OK;
+  int32_t* out = (int32_t*)((char*)g->aux + L.samples);
+  k_samples<<<g->sms * 8, 256, 0, s>>>(g->view.col, g->nnz, out);
+  if (cudaGetLastError() != cudaSuccess) return N2V_ERR_CUDA;
+  g->view.samples = out;
+  return N2V_OK;
+}
+
 // Build (or rebuild) the hub cache under g->tune.  Synchronises the stream.
 static int build_hubs(n2v_graph* g, const AuxLayout& L, cudaStream_t s) {
   g->view.hub_of = nullptr;
@@ -418,7 +446,7 @@ int n2v_graph_load(const int64_t* row_ptr, const int32_t* col, const uint32_t* w
   if (!tune_ok(tt)) return N2V_ERR_INVALID_ARG;
   const int weighted = w ? 1 : 0;
   AuxLayout L = aux_layout(n, nnz, weighted, tt);
-  if (aux_bytes < L.total) return N2V_ERR_NO_MEM;
+  if (aux_bytes < L.samples) return N2V_ERR_NO_MEM;
   cudaStream_t s = (cudaStream_t)stream;
 
   n2v_graph* g = (n2v_graph*)calloc(1, sizeof(n2v_graph));
@@ -467,8 +495,11 @@ int n2v_graph_load(const int64_t* row_ptr, const int32_t* col, const uint32_t* w
     g->info.w_min = weighted && nnz > 0 ? 0xffffffffu - (uint32_t)sc[kScWMin] : 1u;
     g->info.w_max = weighted && nnz > 0 ? (uint32_t)sc[kScWMax] : 1u;
     for (int i = 0; i < 34; ++i) g->info.deg_hist[i] = (int64_t)sc[kScHist + i];
-    rc = build_hubs(g, L, s);
+    rc = build_samples(g, L, s);
+    if (rc == N2V_OK) rc = build_hubs(g, L, s);
     if (rc == N2V_OK) rc = build_bitmaps(g, L, s);
+    // the samples are read by launches on any stream
+    if (rc == N2V_OK && cudaStreamSynchronize(s) != cudaSuccess) rc = N2V_ERR_CUDA;
   }
   if (rc == N2V_OK) {
     g->graph_cache = new_graph_cache();
@@ -491,7 +522,7 @@ int n2v_graph_info_get(const n2v_graph* g, n2v_graph_info* info) {
 int n2v_graph_retune(n2v_graph* g, const n2v_tune* t, void* stream) {
   if (!g || !t || !tune_ok(*t)) return N2V_ERR_INVALID_ARG;
   AuxLayout L = aux_layout(g->n, g->nnz, g->weighted, *t);
-  if (L.total > g->aux_bytes) return N2V_ERR_NO_MEM;
+  if (L.samples > g->aux_bytes) return N2V_ERR_NO_MEM;
   clear_graph_cache(g);
   const bool same_hubs = t->hub_count == g->tune.hub_count && t->hub_min_degree == g->tune.hub_min_degree &&
                          t->hub_budget_mb == g->tune.hub_budget_mb;

@@ -83,6 +83,9 @@ struct GraphView {
   int64_t bm_min_deg;                    // smallest degree of a bitmap hub
   uint32_t bm_bits;
   uint32_t* status;                      // the graph's device status word (self-checks)
+  // n2v_blocks.cuh: samples[i] = col[8 i], i < ceil(nnz / 8), then from the next multiple of
+  // four on a copy of the block that the end of col cuts; null = none
+  const int32_t* __restrict__ samples;
 };
 
 // One walk job slice, as every sampler sees it.
@@ -122,19 +125,25 @@ struct LaunchCfg {
   size_t l2_persist_bytes;  // bytes at the start of col marked persisting in L2 (0: off)
 };
 
-// Instances of the persistent kernels.  The lean ones run exact walks without
-// hub caches or the merge form, so that the step they inline carries only the
-// probe and staged generators (fewer live registers, fewer spills);
-// kPersistLeanUnw is for graphs without weights and knows that at compile time.
-enum PersistKind { kPersistFull = 0, kPersistLean = 1, kPersistLeanUnw = 2 };
+// Instances of the persistent kernels.  kPersistBlocks steps through sampled
+// blocks (n2v_blocks.cuh).  The others enumerate the specials of a step from the
+// two lists: the lean ones run exact walks without hub caches or the merge form, so
+// that the step they inline carries only the probe and staged generators (fewer
+// live registers, fewer spills).  The Unw kinds are for graphs without weights and
+// know that at compile time.
+enum PersistKind { kPersistFull = 0, kPersistLean = 1, kPersistLeanUnw = 2, kPersistBlocks = 3, kPersistBlocksUnw = 4 };
 
-// The instance an exact-walk launch under L over graph view g can take.
-__host__ __forceinline__ int persist_kind(const LaunchCfg& L, const GraphView& g) {
+// The instance a launch under L over graph view g takes: hub caches and the merge
+// form, when the tuning asks for them, are only in the full one; the blocks
+// serve every other launch on a graph that has its samples, FN-Approx too.
+__host__ __forceinline__ int persist_kind(const LaunchCfg& L, const GraphView& g, bool approx) {
   if (L.merge_ratio != 0 || g.hub_of != nullptr || g.bm_data != nullptr) return kPersistFull;
+  if (g.samples) return g.w ? kPersistBlocks : kPersistBlocksUnw;
+  if (approx) return kPersistFull;
   return g.w ? kPersistLean : kPersistLeanUnw;
 }
 
-// Inside a kPersistLeanUnw kernel: the view's weights are null already (the
+// Inside the kernel of an Unw kind: the view's weights are null already (the
 // host picks that instance only then); stating it lets the compiler drop the
 // weighted code paths.
 __device__ __forceinline__ void fold_unweighted(GraphView& g) {
@@ -282,6 +291,15 @@ __device__ __forceinline__ uint64_t warp_incl_scan_u64(uint64_t x, int lane) {
   return x;
 }
 
+__device__ __forceinline__ uint32_t warp_incl_scan_u32(uint32_t x, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    uint32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
 // First index j in [lo, hi] with a[j] > key, given a non-decreasing a and
 // a[hi] > key.  Whole warp, 32-ary search.
 __device__ __forceinline__ int64_t warp_first_above_u64(const uint64_t* __restrict__ a, int64_t lo,
@@ -371,7 +389,8 @@ __device__ __forceinline__ int32_t bm_pos(const GraphView& g, int32_t h, int32_t
 
 // Layout of the caller's auxiliary buffer (byte offsets, 256-aligned).
 struct AuxLayout {
-  size_t status, scratch, wpre, hub_of, hub_off, hub_bits, hub_vtx, hub_slot, bm_tab, bm_vtx, bm_data, total;
+  size_t status, scratch, wpre, hub_of, hub_off, hub_bits, hub_vtx, hub_slot, bm_tab, bm_vtx, bm_data;
+  size_t samples, total;  // the samples of col last: `samples` bytes are enough for all the rest
   int64_t hubs_cap, slots_cap, bm_cap, bm_words;
   uint32_t bm_bits;
 };

@@ -16,7 +16,7 @@
 #include <mutex>
 #include <vector>
 
-#include "n2v_step.cuh"
+#include "n2v_blocks.cuh"
 
 namespace n2v {
 
@@ -41,12 +41,14 @@ template <int KIND>
 __global__ void __launch_bounds__(kPersistThreads, 5)
     k_serve(GraphView g, const DevSlice* __restrict__ slices, int nslices, int64_t total_slots,
             unsigned long long* __restrict__ counter, LaunchCfg L, uint32_t* __restrict__ spill, uint32_t* status) {
-  if (KIND == kPersistLeanUnw) fold_unweighted(g);
+  constexpr bool BLOCKS = KIND == kPersistBlocks || KIND == kPersistBlocksUnw;
+  if (KIND == kPersistLeanUnw || KIND == kPersistBlocksUnw) fold_unweighted(g);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
-  WarpSmem sm = warp_smem(smem_raw, warp, L, spill ? spill + gw * (int64_t)L.spill_specials : nullptr);
-  warp_smem_init(sm, lane);
+  WarpSmem sm = warp_smem(smem_raw, BLOCKS ? 0 : warp, L, spill ? spill + gw * (int64_t)L.spill_specials : nullptr);
+  if (!BLOCKS) warp_smem_init(sm, lane);
+  uint32_t* rec = (uint32_t*)smem_raw + warp * block_smem_words(L);
   while (!sm.timed_out) {
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(counter, 32ull);
@@ -75,6 +77,7 @@ __global__ void __launch_bounds__(kPersistThreads, 5)
         atomicOr(status, kStInvalidArg);
       }
     }
+    const StepArgs A{S.a_p, S.a_q, ~0ull / (uint64_t)S.a_q, S.seed};
     int k = 0;
     for (; k < S.l; ++k) {
       if (sm.timed_out || !__any_sync(kFull, alive)) break;
@@ -83,8 +86,13 @@ __global__ void __launch_bounds__(kPersistThreads, 5)
       J.a_p = S.a_p;
       J.a_q = S.a_q;
       J.approx = 0;
-      const int32_t x = warp_binned_step<KIND == kPersistFull>(g, alive, t, v, k, (uint64_t)wid, J, L.thread_max_deg,
-                                                               sm, L.stream_ratio, lane);
+      int32_t x;
+      if (BLOCKS)
+        x = blocks_step<KIND == kPersistBlocks>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec,
+                                            block_records(L), lane);
+      else
+        x = warp_binned_step<KIND == kPersistFull>(g, alive, t, v, k, (uint64_t)wid, J, L.thread_max_deg, sm,
+                                                   L.stream_ratio, lane);
       if (mine) row[k] = alive ? x : -1;
       if (alive) {
         if (x < 0) {
@@ -356,10 +364,14 @@ int n2v_serve_step(n2v_server* s, int* launched) {
     return N2V_ERR_CUDA;
   LaunchCfg L = resolve_launch(s->g, N2V_PERSISTENT);
   L.spill_specials = s->cfg.spill_specials;
-  const int smem = (L.block_threads / 32) * warp_smem_bytes(L);
-  const int kind = persist_kind(L, s->g->view);
-  auto kern = kind == kPersistLeanUnw ? k_serve<kPersistLeanUnw> : kind == kPersistLean ? k_serve<kPersistLean>
-                                                                                         : k_serve<kPersistFull>;
+  const int kind = persist_kind(L, s->g->view, false);
+  const bool blocks = kind == kPersistBlocks || kind == kPersistBlocksUnw;
+  const int smem = (L.block_threads / 32) * (blocks ? block_smem_words(L) * 4 : warp_smem_bytes(L));
+  auto kern = kind == kPersistBlocksUnw   ? k_serve<kPersistBlocksUnw>
+              : kind == kPersistBlocks    ? k_serve<kPersistBlocks>
+              : kind == kPersistLeanUnw ? k_serve<kPersistLeanUnw>
+              : kind == kPersistLean    ? k_serve<kPersistLean>
+                                        : k_serve<kPersistFull>;
   if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   kern<<<L.blocks, L.block_threads, smem, s->stream>>>(s->g->view, (const DevSlice*)table, (int)s->host_slices.size(),
                                                        slots, counter, L, spill, s->g->status);

@@ -10,7 +10,7 @@
 #include <new>
 #include <vector>
 
-#include "n2v_step.cuh"
+#include "n2v_blocks.cuh"
 
 namespace n2v {
 
@@ -152,6 +152,57 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
   if (sm.timed_out && lane == 0) atomicOr(J.status, kStTimeout);
 }
 
+// Persistent through sampled blocks: the same loop with blocks_step.
+template <int MINB, bool W>
+__global__ void __launch_bounds__(kPersistThreads, MINB)
+    k_persistent_smp(GraphView g, WalkJob J, unsigned long long* __restrict__ counter, LaunchCfg L,
+                      uint32_t* __restrict__) {
+  if (!W) fold_unweighted(g);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t* rec = (uint32_t*)smem_raw + warp * block_smem_words(L);
+  const StepArgs A{J.a_p, J.a_q, ~0ull / (uint64_t)J.a_q, J.seed};
+  for (;;) {
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(counter, 32ull);
+    base = __shfl_sync(kFull, base, 0);
+    if ((int64_t)base >= J.count) break;
+    const int64_t i = (int64_t)base + lane;
+    const bool mine = i < J.count;
+    const int64_t wid = J.walk_begin + i;
+    int32_t* row = J.walks + i * (int64_t)J.l;
+    int64_t t = -1, v = -1;
+    bool alive = false;
+    if (mine) {
+      const int64_t s0 = J.starts[wid % J.n_starts];
+      if (s0 >= 0 && s0 < g.n) {
+        v = s0;
+        alive = true;
+      } else {
+        atomicOr(J.status, kStInvalidArg);
+      }
+    }
+    int k = 0;
+    for (; k < J.l; ++k) {
+      if (!__any_sync(kFull, alive)) break;
+      const int32_t x =
+          blocks_step<W>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec, block_records(L), lane);
+      N2V_CHECK(g, !alive || (x >= -1 && x < g.n));
+      if (mine) row[k] = alive ? x : -1;
+      if (alive) {
+        if (x < 0) {
+          alive = false;
+        } else {
+          t = v;
+          v = x;
+        }
+      }
+    }
+    if (mine)
+      for (int kk = k; kk < J.l; ++kk) row[kk] = -1;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Persistent with a block tier: each block takes 128 walkers at a time and
 // advances them together, one step at a time; every step is binned into the
@@ -286,6 +337,22 @@ static const void* persistent_fn(int minb, bool blk, int kind) {
       default: return (const void*)k_persistent_blk<5>;
     }
   }
+  if (kind == kPersistBlocksUnw) {
+    switch (minb) {
+      case 4: return (const void*)k_persistent_smp<4, false>;
+      case 6: return (const void*)k_persistent_smp<6, false>;
+      case 8: return (const void*)k_persistent_smp<8, false>;
+      default: return (const void*)k_persistent_smp<5, false>;
+    }
+  }
+  if (kind == kPersistBlocks) {
+    switch (minb) {
+      case 4: return (const void*)k_persistent_smp<4, true>;
+      case 6: return (const void*)k_persistent_smp<6, true>;
+      case 8: return (const void*)k_persistent_smp<8, true>;
+      default: return (const void*)k_persistent_smp<5, true>;
+    }
+  }
   if (kind == kPersistLeanUnw) {
     switch (minb) {
       case 4: return (const void*)k_persistent<4, kPersistLeanUnw>;
@@ -311,12 +378,32 @@ static const void* persistent_fn(int minb, bool blk, int kind) {
 }
 
 // The instance a persistent launch takes: block batches when the block tier is
-// on; else a lean instance unless the call needs FN-Approx, the graph's view
-// carries a hub cache, or the merge form is on (the unweighted one for a graph
-// without weights).
+// on, else the one persist_kind names.
+static int launch_kind(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
+  return L.block_min_deg > 0 ? kPersistFull : persist_kind(L, g, J.approx != 0);
+}
+// Resident 128-thread blocks per SM of the sampled-block instances when the tuning
+// names none.
+constexpr int kBlockStepPerSm = 6;
+
+// The sampled-block instances use no spill area and a quarter of the shared memory,
+// so their grid is their own: the tuning's resident warps per SM, or 24.
+static void block_step_grid(const n2v_graph* g, LaunchCfg& L) {
+  const int warps = g->tune.blocks_per_sm * (g->tune.block_threads / 32);
+  int per_sm = warps > 0 ? (warps + 3) / 4 : kBlockStepPerSm;
+  const int smem = (L.block_threads / 32) * block_smem_words(L) * 4;
+  per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
+  L.minb = persistent_minb(per_sm);
+  L.blocks = g->sms * std::min(per_sm, 8);
+}
+
 static const void* persistent_fn(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
-  const bool blk = L.block_min_deg > 0;
-  return persistent_fn(L.minb, blk, blk || J.approx ? kPersistFull : persist_kind(L, g));
+  return persistent_fn(L.minb, L.block_min_deg > 0, launch_kind(L, g, J));
+}
+// Its dynamic shared memory.
+static int persistent_smem(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
+  return launch_kind(L, g, J) >= kPersistBlocks ? (L.block_threads / 32) * block_smem_words(L) * 4
+                                                   : smem_per_block(L);
 }
 
 // One persistent launch.  With L.l2_persist_bytes > 0 (warp batches only) the
@@ -461,7 +548,7 @@ static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) 
     for (int k = 0; k < c.l; ++k) k_plain_step<<<blocks, 256, 0, s>>>(g->view, J, k);
     return cudaGetLastError();
   }
-  const LaunchCfg L = resolve_launch(g, base);
+  LaunchCfg L = resolve_launch(g, base);
   const int smem = smem_per_block(L);
   if (base == N2V_BINNED) {
     if (smem > 48 * 1024) cudaFuncSetAttribute(k_binned_step, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -473,8 +560,10 @@ static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) 
     return cudaGetLastError();
   }
   // persistent
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, L);
+  const int psmem = persistent_smem(L, g->view, J);
+  if (psmem > 48 * 1024)
+    cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, psmem);
   const int64_t chunks = n_chunks(g, c.count);
   unsigned long long* counters = (unsigned long long*)c.ws;
   cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * (size_t)chunks, s);
@@ -487,7 +576,7 @@ static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) 
     Jc.walk_begin = c.walk_begin + lo;
     Jc.count = std::min<int64_t>(per, c.count - lo);
     Jc.walks = c.walks + lo * (int64_t)c.l;
-    launch_persistent(L, smem, s, g->view, Jc, counters + ci, spill);
+    launch_persistent(L, psmem, s, g->view, Jc, counters + ci, spill);
   }
   return cudaGetLastError();
 }
@@ -837,7 +926,6 @@ extern "C" int n2v_walk_noalloc(const n2v_graph* g, const int32_t* starts, int64
   if (rc != N2V_OK) return rc;
 
   LaunchCfg L = resolve_launch(g, N2V_PERSISTENT);
-  const int smem = smem_per_block(L);
   // the spill area is whatever the scratch has left, shared evenly by the warps
   const int64_t warps = (int64_t)L.blocks * (L.block_threads / 32);
   const int64_t per_warp = (int64_t)((kNoAllocScratchBytes - kNoAllocCounterBytes) / sizeof(uint32_t)) / warps;
@@ -862,6 +950,8 @@ extern "C" int n2v_walk_noalloc(const n2v_graph* g, const int32_t* starts, int64
   J.approx_popular = 0;
   J.w_min = g->info.w_min;
   J.w_max = g->info.w_max;
+  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, L);
+  const int smem = persistent_smem(L, g->view, J);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   const int64_t per = chunks == 1 ? walk_count : g->tune.chunk_walkers;
