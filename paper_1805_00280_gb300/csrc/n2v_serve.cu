@@ -20,15 +20,14 @@
 
 namespace n2v {
 
-// One job's share of a tick, padded in the slot space to a multiple of 32 so
-// that every warp batch belongs to one job.
+// One job's share of a tick: a range of the tick's slots, one for each walker.
 struct DevSlice {
   const int32_t* starts;
   int32_t* walks;       // the job's [n_starts][l] rows
   int64_t n_starts;
   int64_t walk_begin;   // first walk id of this share
   int64_t count;
-  int64_t slot_begin;   // prefix in the tick's slot space (multiple of 32)
+  int64_t slot_begin;   // prefix in the tick's slot space
   uint64_t seed;
   int32_t l;
   uint32_t a_p, a_q;
@@ -50,61 +49,71 @@ __global__ void __launch_bounds__(kPersistThreads, 5)
   if (!BLOCKS) warp_smem_init(sm, lane);
   uint32_t* rec = (uint32_t*)smem_raw + warp * block_smem_words(L);
   while (!sm.timed_out) {
+    int take = 32;
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(counter, 32ull);
+    if (lane == 0) {
+      if (BLOCKS) take = grab_size(L, total_slots, *(volatile unsigned long long*)counter);
+      base = atomicAdd(counter, (unsigned long long)take);
+    }
     base = __shfl_sync(kFull, base, 0);
+    take = __shfl_sync(kFull, take, 0);
     if ((int64_t)base >= total_slots) break;
-    // the slice holding this batch: last slot_begin <= base
-    int lo = 0, hi = nslices - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (slices[mid].slot_begin <= (int64_t)base) lo = mid;
-      else hi = mid - 1;
-    }
-    const DevSlice S = slices[lo];
-    const int64_t i = (int64_t)base - S.slot_begin + lane;
-    const bool mine = i < S.count;
-    const int64_t wid = S.walk_begin + i;
-    int32_t* row = S.walks + wid * (int64_t)S.l;
-    int64_t t = -1, v = -1;
-    bool alive = false;
-    if (mine) {
-      const int64_t s0 = S.starts[wid % S.n_starts];
-      if (s0 >= 0 && s0 < g.n) {
-        v = s0;
-        alive = true;
-      } else {
-        atomicOr(status, kStInvalidArg);
+    const int64_t end = min((int64_t)base + take, total_slots);
+    // the slices these slots lie in, one after another
+    for (int64_t slot = (int64_t)base; slot < end && !sm.timed_out;) {
+      int lo = 0, hi = nslices - 1;  // the last slice that begins at or before slot
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (slices[mid].slot_begin <= slot) lo = mid;
+        else hi = mid - 1;
       }
-    }
-    const StepArgs A{S.a_p, S.a_q, ~0ull / (uint64_t)S.a_q, S.seed};
-    int k = 0;
-    for (; k < S.l; ++k) {
-      if (sm.timed_out || !__any_sync(kFull, alive)) break;
-      WalkJob J;  // the slice's parameters (serving is exact: no FN-Approx)
-      J.seed = S.seed;
-      J.a_p = S.a_p;
-      J.a_q = S.a_q;
-      J.approx = 0;
-      int32_t x;
-      if (BLOCKS)
-        x = blocks_step<KIND == kPersistBlocks>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec,
-                                            block_records(L), lane);
-      else
-        x = warp_binned_step<KIND == kPersistFull>(g, alive, t, v, k, (uint64_t)wid, J, L.thread_max_deg, sm,
-                                                   L.stream_ratio, lane);
-      if (mine) row[k] = alive ? x : -1;
-      if (alive) {
-        if (x < 0) {
-          alive = false;
+      const DevSlice S = slices[lo];
+      const int64_t i = slot - S.slot_begin + lane;
+      const int64_t here = min(end, S.slot_begin + S.count) - slot;  // slots of this slice: 1 .. 32
+      slot += here;
+      const bool mine = lane < here;
+      const int64_t wid = S.walk_begin + i;
+      int32_t* row = S.walks + wid * (int64_t)S.l;
+      int64_t t = -1, v = -1;
+      bool alive = false;
+      if (mine) {
+        const int64_t s0 = S.starts[wid % S.n_starts];
+        if (s0 >= 0 && s0 < g.n) {
+          v = s0;
+          alive = true;
         } else {
-          t = v;
-          v = x;
+          atomicOr(status, kStInvalidArg);
         }
       }
+      const StepArgs A{S.a_p, S.a_q, ~0ull / (uint64_t)S.a_q, S.seed};
+      int k = 0;
+      for (; k < S.l; ++k) {
+        if (sm.timed_out || !__any_sync(kFull, alive)) break;
+        WalkJob J;  // the slice's parameters (serving is exact: no FN-Approx)
+        J.seed = S.seed;
+        J.a_p = S.a_p;
+        J.a_q = S.a_q;
+        J.approx = 0;
+        int32_t x;
+        if (BLOCKS)
+          x = blocks_step<KIND == kPersistBlocks>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec,
+                                                  block_records(L), lane);
+        else
+          x = warp_binned_step<KIND == kPersistFull>(g, alive, t, v, k, (uint64_t)wid, J, L.thread_max_deg, sm,
+                                                     L.stream_ratio, lane);
+        if (mine) row[k] = alive ? x : -1;
+        if (alive) {
+          if (x < 0) {
+            alive = false;
+          } else {
+            t = v;
+            v = x;
+          }
+        }
+      }
+      if (mine)
+        for (int kk = k; kk < S.l; ++kk) row[kk] = -1;  // after the walk ended
     }
-    if (mine)
-      for (int kk = k; kk < S.l; ++kk) row[kk] = -1;  // after the walk ended
   }
   if (sm.timed_out && lane == 0) atomicOr(status, kStTimeout);
 }
@@ -348,7 +357,7 @@ int n2v_serve_step(n2v_server* s, int* launched) {
     s->host_slices.push_back(d);
     t.shares.push_back({id, take});
     j.launched += take;
-    slots += (take + 31) / 32 * 32;
+    slots += take;
     walkers += take;
   }
   char* table = s->arena + (size_t)s->cur * (sizeof(DevSlice) * (size_t)s->cfg.max_jobs_per_tick + 256);
@@ -364,6 +373,7 @@ int n2v_serve_step(n2v_server* s, int* launched) {
     return N2V_ERR_CUDA;
   LaunchCfg L = resolve_launch(s->g, N2V_PERSISTENT);
   L.spill_specials = s->cfg.spill_specials;
+  L.lane_walks = lane_walks(s->g->info);
   const int kind = persist_kind(L, s->g->view, false);
   const bool blocks = kind == kPersistBlocks || kind == kPersistBlocksUnw;
   const int smem = (L.block_threads / 32) * (blocks ? block_smem_words(L) * 4 : warp_smem_bytes(L));

@@ -163,12 +163,17 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
   uint32_t* rec = (uint32_t*)smem_raw + warp * block_smem_words(L);
   const StepArgs A{J.a_p, J.a_q, ~0ull / (uint64_t)J.a_q, J.seed};
   for (;;) {
+    int take = 32;
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(counter, 32ull);
+    if (lane == 0) {
+      take = grab_size(L, J.count, *(volatile unsigned long long*)counter);
+      base = atomicAdd(counter, (unsigned long long)take);
+    }
     base = __shfl_sync(kFull, base, 0);
+    take = __shfl_sync(kFull, take, 0);
     if ((int64_t)base >= J.count) break;
     const int64_t i = (int64_t)base + lane;
-    const bool mine = i < J.count;
+    const bool mine = lane < take && i < J.count;
     const int64_t wid = J.walk_begin + i;
     int32_t* row = J.walks + i * (int64_t)J.l;
     int64_t t = -1, v = -1;
@@ -395,6 +400,7 @@ static void block_step_grid(const n2v_graph* g, LaunchCfg& L) {
   per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
   L.minb = persistent_minb(per_sm);
   L.blocks = g->sms * std::min(per_sm, 8);
+  L.lane_walks = lane_walks(g->info);
 }
 
 static const void* persistent_fn(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
