@@ -124,6 +124,52 @@ __device__ __forceinline__ uint64_t div_by_aq(const StepArgs& A, uint64_t x) {
 }
 
 // ---------------------------------------------------------------------------
+// One lane, one step whose weights do not depend on N(t): the first step and an
+// approximated one (static weights: t < 0), and every step at q = 1 (a_q is one),
+// where each neighbour but t weighs w alone.  t's index in N(v) takes one binary
+// search (none when p = 1 too), the rest is the static prefix with one jump at t.
+// T and r carry the common factor one = 2^16, which r drops again:
+// floor(floor(u 2^16 W / 2^64) / 2^16) = floor(u W / 2^64).
+// Measured, R-MAT 20, p = q = 1, 51.7M steps: 129 ms through the two lists,
+// 1.2 ms here.
+template <bool W>
+__device__ __forceinline__ int32_t first_order_step(const GraphView& g, int64_t bv, int dv, int32_t t, uint64_t u,
+                                                    uint32_t a_p) {
+  const int32_t* __restrict__ nv = g.col + bv;
+  int pt = dv;  // index of t in N(v), dv when it is not there or weighs like the others
+  if (t >= 0 && a_p != kAlphaOne) {
+    pt = lower_bound32(nv, dv, t);
+    if (pt < dv && __ldg(nv + pt) != t) pt = dv;
+  }
+  uint64_t wt = 0, c0 = 0;  // w(v, t), and C just before t
+  if (pt < dv) {
+    wt = W ? (uint64_t)__ldg(g.w + bv + pt) : 1ull;
+    c0 = (W ? __ldg(g.wpre + bv + pt) - wt : (uint64_t)pt) << 16;
+  }
+  const uint64_t jump = ((uint64_t)a_p - (uint64_t)kAlphaOne) * wt;  // modulo 2^64
+  const uint64_t T = ((W ? __ldg(g.wpre + bv + dv - 1) : (uint64_t)dv) << 16) + jump;
+  if (W && T == 0) return -1;
+  uint64_t r = scale_draw(u, T);
+  if (pt < dv && r >= c0) {
+    if (r - c0 < (uint64_t)a_p * wt) return t;  // inside t's share
+    r -= jump;
+  }
+  const uint64_t m = r >> 16;  // first j with W_j > m
+  if (!W) return __ldg(nv + m);
+  int lo = 0, n = dv;
+  while (n > 0) {
+    const int half = n >> 1;
+    if (__ldg(g.wpre + bv + lo + half) <= m) {
+      lo += half + 1;
+      n -= half + 1;
+    } else {
+      n = half;
+    }
+  }
+  return __ldg(nv + lo);
+}
+
+// ---------------------------------------------------------------------------
 // One lane, one step (k >= 1), 1 <= deg v <= kLaneDeg: each neighbour of v is
 // looked up in N(t), four at a time, and the hits are kept as a bit mask.
 // Thirty-two walkers of a warp go side by side, so a step of 20 neighbours costs
@@ -687,8 +733,8 @@ __device__ __forceinline__ int grab_size(const LaunchCfg& L, int64_t count, unsi
 
 // ---------------------------------------------------------------------------
 // One step of up to 32 walkers, one per lane.  On its lane: the first step, an
-// approximated step and the steps that are short enough; the others one after
-// another by the whole warp.
+// approximated step, every step at q = 1 and the steps that are short enough; the
+// others one after another by the whole warp.
 template <bool W>
 __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, int64_t t, int64_t v, int k, uint64_t wid,
                                                const WalkJob& J, const StepArgs& A, int thr, uint32_t* rec, int cap,
@@ -702,15 +748,17 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
   if (alive) {
     bv = g.rp[v];
     dv = (int)(g.rp[v + 1] - bv);
-    if (k > 0) {
+    const bool two = k > 0 && (A.a_q != kAlphaOne || J.approx);  // N(t) plays a part
+    if (two) {
       bt = g.rp[t];
       dt = (int)(g.rp[t + 1] - bt);
     }
     u = philox_draw(A.seed, wid, (uint32_t)k);
+    const bool fixed = k == 0 || approx_here(J, k, dv, dt);
     if (dv == 0) {
       // a dead end
-    } else if (k == 0 || approx_here(J, k, dv, dt)) {
-      x = static_step(g, bv, bv + dv, u);
+    } else if (fixed || A.a_q == kAlphaOne) {
+      x = first_order_step<W>(g, bv, dv, fixed ? -1 : (int32_t)t, u, fixed ? kAlphaOne : A.a_p);
     } else if (dv <= min(thr, kLaneDeg)) {
       how = kLane;
     } else {

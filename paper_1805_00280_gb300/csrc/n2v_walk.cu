@@ -393,14 +393,14 @@ constexpr int kBlockStepPerSm = 6;
 
 // The sampled-block instances use no spill area and a quarter of the shared memory,
 // so their grid is their own: the tuning's resident warps per SM, or 24.
-static void block_step_grid(const n2v_graph* g, LaunchCfg& L) {
+static void block_step_grid(const n2v_graph* g, const WalkJob& J, LaunchCfg& L) {
   const int warps = g->tune.blocks_per_sm * (g->tune.block_threads / 32);
   int per_sm = warps > 0 ? (warps + 3) / 4 : kBlockStepPerSm;
   const int smem = (L.block_threads / 32) * block_smem_words(L) * 4;
   per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
   L.minb = persistent_minb(per_sm);
   L.blocks = g->sms * std::min(per_sm, 8);
-  L.lane_walks = lane_walks(g->info);
+  L.lane_walks = J.a_q == kAlphaOne || lane_walks(g->info);
 }
 
 static const void* persistent_fn(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
@@ -566,7 +566,7 @@ static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) 
     return cudaGetLastError();
   }
   // persistent
-  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, L);
+  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, J, L);
   const int psmem = persistent_smem(L, g->view, J);
   if (psmem > 48 * 1024)
     cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, psmem);
@@ -956,7 +956,7 @@ extern "C" int n2v_walk_noalloc(const n2v_graph* g, const int32_t* starts, int64
   J.approx_popular = 0;
   J.w_min = g->info.w_min;
   J.w_max = g->info.w_max;
-  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, L);
+  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, J, L);
   const int smem = persistent_smem(L, g->view, J);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
