@@ -46,8 +46,8 @@ __device__ __forceinline__ BlockRow block_row(const GraphView& g, int64_t b, int
   r.n1 = (int)(((b + d - 1) >> 3) - f);
   r.head = (int)(b & 7);
   r.len = d;
-  r.cut = 8 * (f + r.n1 + 1) > g.nnz ? r.n1 : -1;
-  r.tail = g.samples + ((g.nnz + 31) >> 5 << 2);
+  r.cut = f + r.n1 == g.cut_block ? r.n1 : -1;
+  r.tail = g.tail;
   return r;
 }
 
@@ -319,7 +319,10 @@ struct BlockStep {
 #pragma unroll
     for (int e = 0; e < 4; ++e) asm volatile("ld.shared.s32 %0, [%1+%2];" : "=r"(s[e]) : "r"(p[e]), "n"(4 * (ST - 1)));
 #pragma unroll
-    for (int e = 0; e < 4; ++e) p[e] += s[e] <= x[e] ? 4u * ST : 0u;
+    for (int e = 0; e < 4; ++e)
+      asm("{\n .reg .pred q;\n setp.le.s32 q, %1, %2;\n @q add.u32 %0, %0, %3;\n}"
+          : "+r"(p[e])
+          : "r"(s[e]), "r"(x[e]), "n"(4 * ST));
   }
 
   // State of a pass over the keys.
@@ -529,6 +532,23 @@ struct BlockStep {
     __syncwarp();
     return W ? (Sum)wx : (Sum)__popc(word);
   }
+
+#ifdef N2V_STATS
+  // As the generator modes of warp_step: keys searched in global memory (0, 1), or in staged
+  // samples (2, 3); keys N(v) are modes 0 and 3.
+  __device__ __forceinline__ void stat(long long t_enter) const {
+    const bool vk = dv <= dt;
+    const int sh = vk ? dv : dt, lg = vk ? dt : dv;
+    const bool staged = sh > 32 && (lg >> 3) <= 400 * ((sh + 127) >> 7);
+    const int m = staged ? (vk ? 3 : 2) : (vk ? 0 : 1);
+    if (lane == 0) {
+      N2V_STAT(kStatMode + 4 * m, 1);
+      N2V_STAT(kStatMode + 4 * m + 1, clock64() - t_enter);
+      N2V_STAT(kStatMode + 4 * m + 2, sh);
+      N2V_STAT(kStatMode + 4 * m + 3, lg);
+    }
+  }
+#endif
 
   // The chosen position in N(v), or -1 when T == 0.
   __device__ __forceinline__ int run(uint64_t u) {
@@ -745,6 +765,9 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
   uint64_t u = 0;
   int64_t bv = 0, bt = 0;
   int dv = 0, dt = 0;
+#ifdef N2V_STATS
+  const long long t_lane = clock64();
+#endif
   if (alive) {
     bv = g.rp[v];
     dv = (int)(g.rp[v + 1] - bv);
@@ -772,6 +795,16 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
     how = kDone;
   }
   __syncwarp();
+#ifdef N2V_STATS
+  {
+    const unsigned mx = __reduce_max_sync(kFull, (unsigned)min(clock64() - t_lane, 0xffffffffll));
+    const bool any_alive = __any_sync(kFull, alive);  // every lane votes
+    if (lane == 0 && any_alive) {
+      N2V_STAT(k == 0 ? kStatFirst : kStatLaneSteps, 1);
+      N2V_STAT(k == 0 ? kStatFirstCycles : kStatLaneCycles, mx);
+    }
+  }
+#endif
   unsigned wm = __ballot_sync(kFull, how != kDone);
   while (wm) {
     const int src = __ffs(wm) - 1;
@@ -789,7 +822,13 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
                     cap,
                     g.col + bv_,
                     g.col + bt_};
+#ifdef N2V_STATS
+    const long long t_enter = clock64();
+#endif
     const int j = st.run(__shfl_sync(kFull, u, src));
+#ifdef N2V_STATS
+    st.stat(t_enter);
+#endif
     if (lane == src) x = j < 0 ? -1 : __ldg(g.col + bv + j);
     __syncwarp();
   }

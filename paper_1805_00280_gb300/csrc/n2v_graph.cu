@@ -315,6 +315,8 @@ static int build_samples(n2v_graph* g, const AuxLayout& L, cudaStream_t s) {
   k_samples<<<g->sms * 8, 256, 0, s>>>(g->view.col, g->nnz, out);
   if (cudaGetLastError() != cudaSuccess) return N2V_ERR_CUDA;
   g->view.samples = out;
+  g->view.tail = out + ((g->nnz + 31) >> 5 << 2);
+  g->view.cut_block = g->nnz & 7 ? g->nnz >> 3 : -1;
   return N2V_OK;
 }
 

@@ -83,9 +83,11 @@ struct GraphView {
   int64_t bm_min_deg;                    // smallest degree of a bitmap hub
   uint32_t bm_bits;
   uint32_t* status;                      // the graph's device status word (self-checks)
-  // n2v_blocks.cuh: samples[i] = col[8 i], i < ceil(nnz / 8), then from the next multiple of
-  // four on a copy of the block that the end of col cuts; null = none
+  // n2v_blocks.cuh: samples[i] = col[8 i], i < ceil(nnz / 8) (null = none), and a copy of the
+  // block that the end of col cuts (cut_block, or -1)
   const int32_t* __restrict__ samples;
+  const int32_t* __restrict__ tail;
+  int64_t cut_block;
 };
 
 // One walk job slice, as every sampler sees it.

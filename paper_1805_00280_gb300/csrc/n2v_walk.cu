@@ -162,6 +162,9 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t* rec = (uint32_t*)smem_raw + warp * block_smem_words(L);
   const StepArgs A{J.a_p, J.a_q, ~0ull / (uint64_t)J.a_q, J.seed};
+#ifdef N2V_STATS
+  const long long t_kernel = clock64();
+#endif
   for (;;) {
     int take = 32;
     unsigned long long base = 0;
@@ -206,6 +209,9 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
     if (mine)
       for (int kk = k; kk < J.l; ++kk) row[kk] = -1;
   }
+#ifdef N2V_STATS
+  if (lane == 0) N2V_STAT(kStatKernelCycles, clock64() - t_kernel);
+#endif
 }
 
 // ---------------------------------------------------------------------------
