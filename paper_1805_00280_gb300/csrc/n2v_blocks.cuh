@@ -64,26 +64,19 @@ __device__ __forceinline__ Block block_load(const BlockRow& r, int i) {
   return block_at(i == r.cut ? r.tail : r.blk + 8ll * i);
 }
 
-// Drop the entries of block i that belong to other rows (only the row's first and
-// last blocks have some).
-__device__ __forceinline__ void block_trim(const BlockRow& r, int i, Block& b) {
-  const unsigned at = (unsigned)(8 * i - r.head);
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-    if (at + j >= (unsigned)r.len) b.s[j] = -1;
-}
-
 __device__ __forceinline__ bool block_has(const Block& b, int32_t x) {
   return b.s[0] == x || b.s[1] == x || b.s[2] == x || b.s[3] == x || b.s[4] == x || b.s[5] == x || b.s[6] == x ||
          b.s[7] == x;
 }
 
-// Position in the row of an x that the (trimmed) block i holds.
+// Position in the row of an x that block i holds as the row's own.
 __device__ __forceinline__ int block_pos(const BlockRow& r, int i, const Block& b, int32_t x) {
-  int p = 7;
+  const unsigned at = (unsigned)(8 * i - r.head);
+  unsigned p = 0;
 #pragma unroll
-  for (int j = 6; j >= 0; --j) p = b.s[j] == x ? j : p;
-  return 8 * i - r.head + p;
+  for (int j = 0; j < 8; ++j)
+    if (b.s[j] == x && at + j < (unsigned)r.len) p = at + j;
+  return (int)p;
 }
 
 // First position of the row whose entry is >= x, given the block of x (the number
@@ -116,12 +109,6 @@ struct StepArgs {
   uint64_t inv_q;  // floor((2^64 - 1) / a_q)
   uint64_t seed;
 };
-
-__device__ __forceinline__ uint64_t div_by_aq(const StepArgs& A, uint64_t x) {
-  uint64_t q = __umul64hi(x, A.inv_q);
-  if (x - q * (uint64_t)A.a_q >= (uint64_t)A.a_q) ++q;  // the estimate is the quotient or one less
-  return q;
-}
 
 // ---------------------------------------------------------------------------
 // One lane, one step whose weights do not depend on N(t): the first step and an
@@ -195,12 +182,19 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
       block_search<4>(rt, 0, x, node);
 #pragma unroll
       for (int e = 0; e < 4; ++e) b[e] = block_load(rt, node[e]);
-      uint32_t m = 0;
+      uint32_t m = 0, check = 0;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        block_trim(rt, node[e], b[e]);
-        m |= block_has(b[e], x[e]) ? 1u << e : 0u;
+        if (block_has(b[e], x[e])) m |= 1u << e;
+        if (node[e] == 0 || node[e] == rt.n1) check |= 1u << e;
         if (x[e] == t) pt = min(pt, i0 + e);
+      }
+#pragma unroll 1
+      for (check &= m; check; check &= check - 1) {  // perhaps a neighbouring row's entry
+        const int e = __ffs(check) - 1;
+        const int32_t y = __ldg(nv + min(i0 + e, dv - 1));
+        const int p = lower_bound32(g.col + bt, dt, y);
+        if (p >= dt || __ldg(g.col + bt + p) != y) m &= ~(1u << e);
       }
       hits |= (uint64_t)m << i0;
     }
@@ -267,18 +261,28 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
 //
 // t itself (weight 1/p) is never counted as a hit: its part of D is added where
 // a position is at or behind it.
+//
+// Bound: instruction issue while the graph's hot lists stay in L2, DRAM beyond.  The
+// size of the code is part of it, since the warps of an SM are all over it: at 2,500
+// instructions a kernel waits for none, at 3,300 a seventh of the time, at 4,600 it
+// takes twice as long (R-MAT 20).  A separate form for one batch in registers saved a
+// fifth of WeC-20's instructions and was slower for that reason.
 constexpr int kWin = 512;         // staged samples per warp
 constexpr int32_t kNoKey = -2;    // in the place of a key past the end: below every vertex, equal to none
 
 // Shared memory of one warp: cap record words, cap more (the blocks of the first
 // keys; with weights the records take both), kWin samples.
 __host__ __device__ __forceinline__ int block_records(const LaunchCfg& L) {
-  return L.smem_specials < 1024 ? L.smem_specials : 1024;
+  return L.smem_specials < 256 ? L.smem_specials : 256;
 }
 __host__ __device__ __forceinline__ int block_smem_words(const LaunchCfg& L) { return 2 * block_records(L) + kWin; }
 
 template <bool W>
 struct BlockStep {
+  // Chunks of a batch.  With weights two: four are 4,200 instructions and 300 bytes of spills,
+  // and weighted R-MAT 23 takes 160 ms instead of 143 ms; without, two cost R-MAT 24 133 ms
+  // instead of 117 ms.
+  static constexpr int kB = W ? 2 : 4;
   using Sum = typename std::conditional<W, uint64_t, uint32_t>::type;  // of hits, or of their weights
   const GraphView& g;
   const StepArgs& A;
@@ -308,21 +312,89 @@ struct BlockStep {
   __device__ __forceinline__ uint64_t w_before(int p) const {
     return W ? (p > 0 ? __ldg(g.wpre + bv + p - 1) : 0ull) : (uint64_t)p;
   }
+  // a_q times it
+  __device__ __forceinline__ uint64_t base_before(int p) const {
+    return W ? (uint64_t)A.a_q * w_before(p) : (uint64_t)A.a_q * (uint32_t)p;
+  }
+  // D of hits that number (weigh) s
+  __device__ __forceinline__ uint64_t part_of(Sum s) const {
+    const int32_t d1 = (int32_t)kAlphaOne - (int32_t)A.a_q;
+    return W ? (uint64_t)(int64_t)d1 * s : (uint64_t)((int64_t)d1 * (int32_t)s);
+  }
+
   // first position in [lo, hi) of N(v) with an entry >= x (hi if none)
   __device__ __forceinline__ int pos_of(int lo, int hi, int32_t x) const { return lo + lower_bound32(nv + lo, hi - lo, x); }
 
   // The search of one staged level: p points at the first staged sample not yet known to
   // be at or below the key.
-  template <int ST>
-  __device__ __forceinline__ static void level(uint32_t (&p)[4], const int32_t (&x)[4]) {
-    int32_t s[4];
+  template <int ST, int NE>
+  __device__ __forceinline__ static void level(uint32_t (&p)[NE], const int32_t (&x)[NE]) {
+    int32_t s[NE];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) asm volatile("ld.shared.s32 %0, [%1+%2];" : "=r"(s[e]) : "r"(p[e]), "n"(4 * (ST - 1)));
+    for (int e = 0; e < NE; ++e) asm volatile("ld.shared.s32 %0, [%1+%2];" : "=r"(s[e]) : "r"(p[e]), "n"(4 * (ST - 1)));
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
+    for (int e = 0; e < NE; ++e)
       asm("{\n .reg .pred q;\n setp.le.s32 q, %1, %2;\n @q add.u32 %0, %0, %3;\n}"
           : "+r"(p[e])
           : "r"(s[e]), "r"(x[e]), "n"(4 * ST));
+  }
+
+  // Number of the first n staged samples (n < kWin, ascending, larger ones behind them) at
+  // or below each key: a search of the 2^d - 1 >= n first slots.
+  template <int NE>
+  __device__ __forceinline__ void search_staged(const int32_t* win, int n, const int32_t (&x)[NE], int (&count)[NE]) const {
+    const uint32_t w0 = smem_addr(win);
+    uint32_t p[NE];
+#pragma unroll
+    for (int e = 0; e < NE; ++e) p[e] = w0;
+    if (n >= 32) {
+      if (n >= 128) {
+        if (n >= 256) level<256>(p, x);
+        level<128>(p, x);
+      }
+      if (n >= 64) level<64>(p, x);
+      level<32>(p, x);
+    }
+    if (n >= 8) {
+      if (n >= 16) level<16>(p, x);
+      level<8>(p, x);
+    }
+    level<4>(p, x);
+    level<2>(p, x);
+    level<1>(p, x);
+#pragma unroll
+    for (int e = 0; e < NE; ++e) count[e] = (int)((p[e] - w0) >> 2);
+  }
+
+  // Compare keys and blocks; the lane's first key is keys[i0], the others 32 apart.  A match in
+  // the row's first or last block may be an entry of a neighbouring row: there the row's own
+  // entries are searched (rare, and one copy of it).
+  template <int NE>
+  __device__ __forceinline__ void match(const BlockRow& r, const int32_t* __restrict__ keys, int i0,
+                                        const int (&node)[NE], const int32_t (&x)[NE], const Block (&bl)[NE],
+                                        bool (&in)[NE]) const {
+    unsigned m = 0, check = g.loops ? 15u : 0u;
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+      in[e] = block_has(bl[e], x[e]);
+      m |= in[e] ? 1u << e : 0u;
+      if (node[e] == 0 || node[e] == r.n1) check |= 1u << e;
+    }
+    check &= m;
+    if (check) {
+      const int32_t* __restrict__ row = r.blk + r.head;
+      unsigned no = 0;
+#pragma unroll 1
+      for (; check; check &= check - 1) {
+        const int e = __ffs(check) - 1;
+        const int32_t y = __ldg(keys + i0 + 32 * e);
+        const int p = lower_bound32(row, r.len, y);
+        // t itself is no hit (only a graph with self-loops has t in N(t))
+        if (p >= r.len || __ldg(row + p) != y || y == t) no |= 1u << e;
+      }
+#pragma unroll
+      for (int e = 0; e < NE; ++e) in[e] = in[e] && !((no >> e) & 1u);
+    }
   }
 
   // State of a pass over the keys.
@@ -334,20 +406,20 @@ struct BlockStep {
     int from;              // samples at or below every key still to come
     int group;             // chunks that share one record (1, or a multiple of four)
     int left, gi;          // of the current group: chunks to come, and its record
-    int32_t nx[4], ns[4];  // the next batch's keys and samples
-    Sum sum, before;       // hits so far, and before the group (with weights: this lane's share of their weights)
     int pt;                // index of the key equal to t that this lane saw, or -1
+    int32_t nx[kB], ns[4];  // the next batch's keys and samples
+    Sum sum, before;       // hits so far, and before the group (with weights: this lane's share of their weights)
   };
 
   __device__ __forceinline__ void fetch(Pass& P, const BlockRow& r, int c) const {
     const int32_t* k = P.keys + 32 * c;
     const int n = P.nk - 32 * c;
-    if (n >= 128) {
+    if (n >= 32 * kB) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) P.nx[e] = __ldg(k + 32 * e);
+      for (int e = 0; e < kB; ++e) P.nx[e] = __ldg(k + 32 * e);
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) P.nx[e] = 32 * e < n - lane ? __ldg(k + 32 * e) : kNoKey;
+      for (int e = 0; e < kB; ++e) P.nx[e] = 32 * e < n - lane ? __ldg(k + 32 * e) : kNoKey;
     }
     const int32_t* q = r.smp + P.from + lane;
     const int m = r.n1 - P.from - lane;
@@ -359,16 +431,15 @@ struct BlockStep {
     }
   }
 
-  // One batch: chunks c .. c + 3.
+  // One batch: chunks c .. c + kB - 1.
   __device__ __forceinline__ void batch(Pass& P, const BlockRow& r, int c, bool vk) {
     int32_t* win = (int32_t*)(rec + 2 * cap);
-    int32_t x[4];
-    int node[4];
+    int32_t x[kB];
+    int node[kB];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) x[e] = P.nx[e];
+    for (int e = 0; e < kB; ++e) x[e] = P.nx[e];
     // the batch's largest key
-    const int32_t last = P.nk - 32 * c >= 128 ? __shfl_sync(kFull, x[3], 31) : P.kmax;
-    bool edges = P.from == 0;
+    const int32_t last = P.nk - 32 * c >= 32 * kB ? __shfl_sync(kFull, x[kB - 1], 31) : P.kmax;
     int below = kWin;  // staged samples at or below the last key
     if (P.stage) {
       win[lane] = P.ns[0];
@@ -394,68 +465,41 @@ struct BlockStep {
       __syncwarp();
     }
     if (below < kWin) {
-      // samples at or below each key, by a search of 2^d - 1 >= below staged samples (the ones
-      // past `below` are above every key)
-      const uint32_t w0 = smem_addr(win);
-      uint32_t p[4];
+      search_staged(win, below, x, node);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) p[e] = w0;
-      if (below >= 32) {
-        if (below >= 128) {
-          if (below >= 256) level<256>(p, x);
-          level<128>(p, x);
-        }
-        if (below >= 64) level<64>(p, x);
-        level<32>(p, x);
-      }
-      if (below >= 8) {
-        if (below >= 16) level<16>(p, x);
-        level<8>(p, x);
-      }
-      level<4>(p, x);
-      level<2>(p, x);
-      level<1>(p, x);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) node[e] = P.from + (int)((p[e] - w0) >> 2);
+      for (int e = 0; e < kB; ++e) node[e] += P.from;
       P.from += below;
     } else {
-      block_search<4>(r, P.from, x, node);
-      if (P.nk - 32 * c >= 128) P.from = __shfl_sync(kFull, node[3], 31);
-      else edges = true;  // the last batch
+      block_search<kB>(r, P.from, x, node);
+      P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
     }
-    edges = edges || P.from == r.n1;
-    Block b[4];
+    Block b[kB];
     if (r.cut < 0) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) b[e] = block_at(r.blk + 8ll * node[e]);
+      for (int e = 0; e < kB; ++e) b[e] = block_at(r.blk + 8ll * node[e]);
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) b[e] = block_load(r, node[e]);
+      for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
     }
-    if (32 * (c + 4) < P.nk) fetch(P, r, c + 4);
-    if (x[0] == t || x[1] == t || x[2] == t || x[3] == t) {  // t is no hit
+    if (32 * (c + kB) < P.nk) fetch(P, r, c + kB);
+    bool has_t = false;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (x[e] == t) {
-          P.pt = 32 * (c + e) + lane;
-          x[e] = kNoKey;
-        }
-      }
+    for (int e = 0; e < kB; ++e) has_t = has_t || x[e] == t;
+    if (has_t) {
+#pragma unroll
+      for (int e = 0; e < kB; ++e) P.pt = x[e] == t ? 32 * (c + e) + lane : P.pt;
     }
-    if (edges) {
+    bool in[kB];
+    match(r, P.keys, 32 * c, node, x, b, in);
+    uint32_t word[kB];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) block_trim(r, node[e], b[e]);
-    }
-    uint32_t word[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const bool in = block_has(b[e], x[e]);
-      word[e] = __ballot_sync(kFull, in);
+    for (int e = 0; e < kB; ++e) {
+      word[e] = __ballot_sync(kFull, in[e]);
       if (!W) {
         P.sum += __popc(word[e]);
       } else {
         const int at = vk ? 32 * (c + e) + lane : block_pos(r, node[e], b[e], x[e]);
-        const uint32_t wx = in ? __ldg(g.w + bv + at) : 0u;
+        const uint32_t wx = in[e] ? __ldg(g.w + bv + at) : 0u;
         P.sum += wx;
         if (P.group == 1) {  // this chunk's weights, in two halves that cannot overflow
           const uint64_t cs = (uint64_t)__reduce_add_sync(kFull, wx & 0xffffu) +
@@ -470,15 +514,20 @@ struct BlockStep {
     }
     if (P.group == 1) {
       if (!W && lane == 0) {
-        *(uint4*)(rec + P.gi) = make_uint4(word[0], word[1], word[2], word[3]);
-        *(uint4*)(rec + cap + P.gi) =
-            make_uint4((uint32_t)node[0], (uint32_t)node[1], (uint32_t)node[2], (uint32_t)node[3]);
+        if (kB == 4) {
+          *(uint4*)(rec + P.gi) = make_uint4(word[0], word[1], word[2 % kB], word[3 % kB]);
+          *(uint4*)(rec + cap + P.gi) =
+              make_uint4((uint32_t)node[0], (uint32_t)node[1], (uint32_t)node[2 % kB], (uint32_t)node[3 % kB]);
+        } else {
+          *(uint2*)(rec + P.gi) = make_uint2(word[0], word[1]);
+          *(uint2*)(rec + cap + P.gi) = make_uint2((uint32_t)node[0], (uint32_t)node[1]);
+        }
       }
-      P.gi += 4;
+      P.gi += kB;
     } else {
       if (P.left == P.group && lane == 0) block_of(P.gi) = (uint32_t)node[0];
-      P.left -= 4;
-      if (P.left == 0 || 32 * (c + 4) >= P.nk) {
+      P.left -= kB;
+      if (P.left <= 0 || 32 * (c + kB) >= P.nk) {
         const Sum gs = W ? (Sum)warp_sum_u64(P.sum - P.before) : (Sum)(P.sum - P.before);
         if (lane == 0) put_total(P.gi, gs);
         P.before = P.sum;
@@ -499,7 +548,7 @@ struct BlockStep {
     P.nk = vk ? dv : dt;
     P.kmax = __ldg((vk ? nv : nt) + P.nk - 1);
     // samples beside a batch of 128 keys: sixteen times the ratio of the lists
-    const int beside = r.len >> 3, nb = (P.nk + 127) >> 7;
+    const int beside = r.len >> 3, nb = (P.nk + 32 * kB - 1) / (32 * kB);
     P.stage = beside <= 48 * nb ? 64 : beside <= 400 * nb ? 128 : 0;
     P.from = from;
     P.group = group;
@@ -510,36 +559,28 @@ struct BlockStep {
     P.pt = -1;
     fetch(P, r, c0);
 #pragma unroll 1
-    for (int c = c0; c < c1; c += 4) batch(P, r, c, vk);
+    for (int c = c0; c < c1; c += kB) batch(P, r, c, vk);
     *pt = P.pt;
     return P.sum;
   }
 
-  // The same for at most 32 keys: one a lane, searched in global memory, one record.
-  __device__ __forceinline__ Sum look_up_one(bool vk, const BlockRow& r, int* pt) {
-    const int nk = vk ? dv : dt;
-    int32_t x[1] = {lane < nk ? __ldg((vk ? nv : nt) + lane) : kNoKey};
-    int node[1];
-    block_search<1>(r, 0, x, node);
-    Block b = block_load(r, node[0]);
-    block_trim(r, node[0], b);
-    *pt = x[0] == t ? lane : -1;
-    const bool in = block_has(b, x[0]) && x[0] != t;
-    const uint32_t word = __ballot_sync(kFull, in);
-    uint32_t wx = 0;
-    if (W && in) wx = __ldg(g.w + bv + (vk ? lane : block_pos(r, node[0], b, x[0])));
-    if (lane == 0) rec[W ? 2 : 0] = word;
-    __syncwarp();
-    return W ? (Sum)wx : (Sum)__popc(word);
-  }
+  // Where a search of the hits ends: at the chosen position, or (keys N(t)) at the last hit
+  // with C at or below r just before it, with D up to there.
+  struct Found {
+    int pos;
+    bool chosen;
+    bool hit;  // pos is a hit
+    int pos_t;
+    uint64_t D, t_part, r;
+  };
 
 #ifdef N2V_STATS
   // As the generator modes of warp_step: keys searched in global memory (0, 1), or in staged
   // samples (2, 3); keys N(v) are modes 0 and 3.
   __device__ __forceinline__ void stat(long long t_enter) const {
-    const bool vk = dv <= dt;
+    const bool vk = dv <= max(dt, 128);
     const int sh = vk ? dv : dt, lg = vk ? dt : dv;
-    const bool staged = sh > 32 && (lg >> 3) <= 400 * ((sh + 127) >> 7);
+    const bool staged = (lg >> 3) <= 400 * ((sh + 127) >> 7);
     const int m = staged ? (vk ? 3 : 2) : (vk ? 0 : 1);
     if (lane == 0) {
       N2V_STAT(kStatMode + 4 * m, 1);
@@ -550,93 +591,78 @@ struct BlockStep {
   }
 #endif
 
+  __device__ __forceinline__ uint64_t part_of_t(int pos_t) const {
+    return pos_t >= 0 ? ((uint64_t)A.a_p - (uint64_t)A.a_q) * (W ? (uint64_t)__ldg(g.w + bv + pos_t) : 1ull) : 0ull;
+  }
+
   // The chosen position in N(v), or -1 when T == 0.
   __device__ __forceinline__ int run(uint64_t u) {
-    const uint64_t aq = A.a_q, d1 = (uint64_t)kAlphaOne - aq, d2 = (uint64_t)A.a_p - aq;
-    const bool vk = dv <= dt;
-    const int nk = vk ? dv : dt;
+    // keys N(v) give positions without a search: also when they are the longer list but one batch
+    const bool vk = dv <= max(dt, 32 * kB);
     const BlockRow row = vk ? block_row(g, bt, dt) : block_row(g, bv, dv);
+    const Found f = search(u, vk, row);
+    return f.chosen ? f.pos : behind(f.pos, f.hit, f.D, f.pos_t, f.t_part, f.r);
+  }
+
+  __device__ __forceinline__ Found search(uint64_t u, bool vk, const BlockRow& row) {
+    const int nk = vk ? dv : dt;
+    // t's position in N(v), -1 when it is not there (keys N(v) have it on the way)
+    int pos_t = vk ? -1 : warp_find(t);
     uint64_t t_part = 0;  // (1/p - 1/q) w(v, t) when t is in N(v)
-    int pos_t = -1;       // t's position in N(v), -1 when it is not there
-    if (!vk) {
-      pos_t = warp_find(t);
-      if (pos_t >= 0) t_part = d2 * (W ? (uint64_t)__ldg(g.w + bv + pos_t) : 1ull);
-    }
-    int c0 = 0, c1 = (nk + 31) >> 5;  // the chunks that can hold the answer
-    uint64_t D = 0;                   // the hits' part of D before chunk c0
-    int plo = 0, phi = dv;            // keys N(t): positions of the first keys of c0 and c1
+    int c0 = 0, c1 = (nk + 31) >> 5;           // the chunks that can hold the answer
+    uint64_t D = 0;                            // the hits' part of D before chunk c0
+    int plo = 0, phi = dv;                     // keys N(t): positions of the first keys of c0 and c1
     uint64_t r = 0;
-    int from = 0;                     // samples at or below every key from c0 on
+    int from = 0;                              // samples at or below every key from c0 on
     for (bool first = true;; first = false) {
       const int nc = c1 - c0;
       int group = 1;
       if (nc > records()) group = ((nc + records() - 1) / records() + 3) & ~3;  // (a multiple of a batch)
       const int n = (nc + group - 1) / group;
-      int pt = -1;
-      const Sum part = nk <= 32 ? look_up_one(vk, row, &pt) : look_up(vk, row, from, c0, c1, group, &pt);
+      int pt;
+      const Sum part = look_up(vk, row, from, c0, c1, group, &pt);
       if (first) {
-        if (vk) {
-          pos_t = __reduce_max_sync(kFull, pt);
-          if (pos_t >= 0) t_part = d2 * (W ? (uint64_t)__ldg(g.w + bv + pos_t) : 1ull);
-        }
-        const uint64_t all = W ? warp_sum_u64(part) : (uint64_t)part;
-        const uint64_t T = aq * w_before(dv) + d1 * all + t_part;
-        if (W && T == 0) return -1;
+        if (vk) pos_t = __reduce_max_sync(kFull, pt);
+        t_part = part_of_t(pos_t);
+        const Sum all = W ? (Sum)warp_sum_u64(part) : part;
+        const uint64_t T = base_before(dv) + part_of(all) + t_part;
+        if (W && T == 0) return Found{-1, true};
         r = scale_draw(u, T);
       }
-      // the record that holds the answer: the first whose end lies above r (keys N(v)), or the
-      // last whose first key's position has C at or below r just before it (keys N(t))
+      // the last record that the answer can lie in: C at or below r just before it (keys N(v):
+      // before its first key; keys N(t): before the first position its first key can have)
       int pick = 0, npl = plo, nph = phi;
       uint64_t Dp = D;
-      for (int i0 = 0; i0 < n && n > 1; i0 += 32) {
+      for (int i0 = 0; i0 < n; i0 += 32) {
         const int i = i0 + lane;
         const Sum x = i < n ? total_at(i, group) : (Sum)0;
         const Sum incl = W ? (Sum)warp_incl_scan_u64(x, lane) : (Sum)warp_incl_scan_u32((uint32_t)x, lane);
-        if (vk) {
-          const int pe = min(dv, 32 * (c0 + group * (i + 1)));
-          bool above = false;
-          if (i < n) above = aq * w_before(pe) + D + d1 * incl + (pos_t >= 0 && pos_t < pe ? t_part : 0ull) > r;
-          const unsigned m = __ballot_sync(kFull, above);
-          const Sum all = __shfl_sync(kFull, incl, 31);
-          if (m) {
-            const int f = __ffs(m) - 1;
-            pick = i0 + f;
-            Dp = D + d1 * __shfl_sync(kFull, (Sum)(incl - x), f);
-            break;
-          }
-          D += d1 * all;
-        } else {
-          int p = plo;
-          bool below = i == 0;
-          if (i > 0 && i < n) {
-            const int32_t y = __ldg(nt + 32 * (c0 + group * i));
-            p = block_lower_bound(row, (int)block_of(i), nv, y);
-            below = aq * w_before(p) + D + d1 * (Sum)(incl - x) + (pos_t >= 0 && pos_t < p ? t_part : 0ull) <= r;
-          }
-          const unsigned m = __ballot_sync(kFull, below);
-          const int f = 31 - __clz(m);  // -1: none of these
-          const Sum excl = __shfl_sync(kFull, (Sum)(incl - x), f & 31), all = __shfl_sync(kFull, incl, 31);
-          const int pf = __shfl_sync(kFull, p, f & 31), pn = __shfl_sync(kFull, p, (f + 1) & 31);
-          if (f >= 0) {
-            pick = i0 + f;
-            Dp = D + d1 * excl;
-            npl = pf;
-          }
-          if (f < 31) {  // the next record's first key bounds the answer
-            if (i0 + f + 1 < n) nph = pn;
-            break;
-          }
-          D += d1 * all;
+        int p = plo;
+        bool before = i == 0;
+        if (i > 0 && i < n) {
+          p = 32 * (c0 + group * i);
+          if (!vk) p = block_lower_bound(row, (int)block_of(i), nv, __ldg(nt + p));
+          before = base_before(p) + D + part_of((Sum)(incl - x)) + (pos_t >= 0 && pos_t < p ? t_part : 0ull) <= r;
         }
+        const unsigned m = __ballot_sync(kFull, before);
+        const int f = 31 - __clz(m);  // -1: none of these
+        const Sum excl = __shfl_sync(kFull, (Sum)(incl - x), f & 31), all = __shfl_sync(kFull, incl, 31);
+        const int pf = __shfl_sync(kFull, p, f & 31), pn = __shfl_sync(kFull, p, (f + 1) & 31);
+        if (f >= 0) {
+          pick = i0 + f;
+          Dp = D + part_of(excl);
+          npl = pf;
+        }
+        if (f < 31) {  // the next record's first key bounds the answer
+          if (i0 + f + 1 < n) nph = pn;
+          break;
+        }
+        D += part_of(all);
       }
       D = Dp;
       plo = npl;
       phi = nph;
-      if (group == 1) {
-        const uint32_t word = ballot_at(pick);
-        return vk ? in_chunk_v(c0 + pick, word, D, pos_t, t_part, r)
-                  : in_chunk_t(c0 + pick, word, D, pos_t, t_part, plo, phi, r);
-      }
+      if (group == 1) return in_chunk(vk, c0 + pick, ballot_at(pick), D, pos_t, t_part, plo, phi, r);
       from = (int)block_of(pick);
       c1 = min(c1, c0 + group * (pick + 1));
       c0 += group * pick;
@@ -660,64 +686,58 @@ struct BlockStep {
     return m ? lo + __ffs(m) - 1 : -1;
   }
 
-  // keys N(v): the answer lies in chunk c (hits: word), D before it
-  __device__ __forceinline__ int in_chunk_v(int c, uint32_t word, uint64_t D, int pos_t, uint64_t t_part, uint64_t r) {
-    const uint64_t d1 = (uint64_t)kAlphaOne - (uint64_t)A.a_q;
-    const int i = 32 * c + lane;
-    uint64_t own;
-    if (W) {
-      const uint64_t wx = ((word >> lane) & 1u) ? (uint64_t)__ldg(g.w + bv + i) : 0ull;
-      own = warp_incl_scan_u64(wx, lane);
-    } else {
-      own = (uint64_t)__popc(word & (0xffffffffu >> (31 - lane)));
+  // The chosen position, given that it lies in chunk c of the keys (its hits: word; D before
+  // it), or, keys N(t), in [plo, phi) from the first key of c on.
+  __device__ __forceinline__ Found in_chunk(bool vk, int c, uint32_t word, uint64_t D, int pos_t, uint64_t t_part,
+                                          int plo, int phi, uint64_t r) {
+    const bool hit = (word >> lane) & 1u;
+    int p = 32 * c + lane;
+    bool live = p < dv;
+    if (!vk) {
+      if (hit) p = pos_of(plo, phi, __ldg(nt + p));
+      live = hit;
     }
-    bool above = false;
-    if (i < dv) above = (uint64_t)A.a_q * w_before(i + 1) + D + d1 * own + (pos_t >= 0 && pos_t <= i ? t_part : 0ull) > r;
-    const unsigned m = __ballot_sync(kFull, above);
-    N2V_CHECK(g, m != 0u);
-    return 32 * c + (m ? __ffs(m) - 1 : 0);
+    Sum incl, own = 1;
+    if (W) {
+      own = hit ? (Sum)__ldg(g.w + bv + p) : (Sum)0;
+      incl = (Sum)warp_incl_scan_u64(own, lane);
+    } else {
+      incl = (Sum)__popc(word & (0xffffffffu >> (31 - lane)));
+    }
+    // keys N(v): is C at this key at or below r?  keys N(t): is C just before this hit?
+    const int q = vk ? p + 1 : p;
+    const bool below = live && base_before(q) + D + part_of(vk ? incl : (Sum)(incl - own)) +
+                                       (pos_t >= 0 && pos_t < q ? t_part : 0ull) <= r;
+    const unsigned m = __ballot_sync(kFull, below);
+    const int f = 31 - __clz(m);
+    if (vk) return Found{min(32 * c + f + 1, dv - 1), true};
+    int prev = plo - 1;
+    if (m) {
+      prev = __shfl_sync(kFull, p, f);
+      D += part_of(__shfl_sync(kFull, incl, f));
+    }
+    return Found{prev, false, m != 0u, pos_t, D, t_part, r};
   }
 
-  // keys N(t): the answer lies in [plo, phi), from the first key of chunk c on (hits: word)
-  __device__ __forceinline__ int in_chunk_t(int c, uint32_t word, uint64_t D, int pos_t, uint64_t t_part, int plo,
-                                            int phi, uint64_t r) {
-    const uint64_t aq = A.a_q, d1 = (uint64_t)kAlphaOne - aq;
-    const bool hit = (word >> lane) & 1u;
-    const int32_t y = hit ? __ldg(nt + 32 * c + lane) : 0;
-    const int p = hit ? pos_of(plo, phi, y) : 0;
-    uint64_t incl, own = hit ? 1ull : 0ull;
-    if (W) {
-      own = hit ? (uint64_t)__ldg(g.w + bv + p) : 0ull;
-      incl = warp_incl_scan_u64(own, lane);
-    } else {
-      incl = (uint64_t)__popc(word & (0xffffffffu >> (31 - lane)));
-    }
-    const bool below =
-        hit && aq * w_before(p) + D + d1 * (incl - own) + (pos_t >= 0 && pos_t < p ? t_part : 0ull) <= r;
-    const unsigned m = __ballot_sync(kFull, below);
-    int prev = plo - 1;  // the answer lies behind prev
-    if (m) {
-      const int f = 31 - __clz(m);
-      prev = __shfl_sync(kFull, p, f);
-      D += d1 * __shfl_sync(kFull, incl, f);
-      // the hit itself
-      if (aq * w_before(prev + 1) + D + (pos_t >= 0 && pos_t < prev ? t_part : 0ull) > r) return prev;
-    }
-    // behind prev every weight is the default up to the next hit, but for t
+  // The chosen position, given that it is prev (a hit, if hit) or behind it and before the
+  // next hit, and the hits' part D of D up to there.
+  __device__ __forceinline__ int behind(int prev, bool hit, uint64_t D, int pos_t, uint64_t t_part, uint64_t r) const {
+    if (hit && base_before(prev + 1) + D + (pos_t >= 0 && pos_t < prev ? t_part : 0ull) > r) return prev;
+    // behind prev every weight is the default, but for t
     const bool passed = pos_t >= 0 && pos_t <= prev;
     if (passed) D += t_part;
     int j = first_above(prev, r - D);
     if (pos_t >= 0 && !passed && j >= pos_t) {  // t lies in (prev, j]: nothing before it is above r
-      if (aq * w_before(pos_t + 1) + D + t_part > r) return pos_t;
+      if (base_before(pos_t + 1) + D + t_part > r) return pos_t;
       j = first_above(pos_t, r - D - t_part);
     }
-    N2V_CHECK(g, j >= plo && j < dv);
+    N2V_CHECK(g, j > prev && j < dv);
     return j;
   }
 
   // First position behind prev whose a_q W exceeds x (the last one if none does).
   __device__ __forceinline__ int first_above(int prev, uint64_t x) const {
-    const uint64_t m = div_by_aq(A, x);
+    const uint64_t m = div_by(x, A.a_q, A.inv_q);
     if (W) return (int)warp_first_above_u64(g.wpre + bv, prev + 1, dv - 1, m, lane);
     const int j = m > (uint64_t)(dv - 1) ? dv - 1 : (int)m;
     return min(dv - 1, max(j, prev + 1));
@@ -755,8 +775,8 @@ __device__ __forceinline__ int grab_size(const LaunchCfg& L, int64_t count, unsi
 // One step of up to 32 walkers, one per lane.  On its lane: the first step, an
 // approximated step, every step at q = 1 and the steps that are short enough; the
 // others one after another by the whole warp.
-template <bool W>
-__device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, int64_t t, int64_t v, int k, uint64_t wid,
+template <bool W, bool APPROX>
+__device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, int32_t t, int32_t v, int k, uint64_t wid,
                                                const WalkJob& J, const StepArgs& A, int thr, uint32_t* rec, int cap,
                                                int lane) {
   enum { kDone, kLane, kMid, kWarp };
@@ -771,17 +791,17 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
   if (alive) {
     bv = g.rp[v];
     dv = (int)(g.rp[v + 1] - bv);
-    const bool two = k > 0 && (A.a_q != kAlphaOne || J.approx);  // N(t) plays a part
+    const bool two = k > 0 && (A.a_q != kAlphaOne || APPROX);  // N(t) plays a part
     if (two) {
       bt = g.rp[t];
       dt = (int)(g.rp[t + 1] - bt);
     }
     u = philox_draw(A.seed, wid, (uint32_t)k);
-    const bool fixed = k == 0 || approx_here(J, k, dv, dt);
+    const bool fixed = k == 0 || (APPROX && approx_here(J, k, dv, dt));
     if (dv == 0) {
       // a dead end
     } else if (fixed || A.a_q == kAlphaOne) {
-      x = first_order_step<W>(g, bv, dv, fixed ? -1 : (int32_t)t, u, fixed ? kAlphaOne : A.a_p);
+      x = first_order_step<W>(g, bv, dv, fixed ? -1 : t, u, fixed ? kAlphaOne : A.a_p);
     } else if (dv <= min(thr, kLaneDeg)) {
       how = kLane;
     } else {
@@ -791,7 +811,7 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
   // steps of up to kLaneDeg neighbours stay on their lanes when enough lanes have one
   const bool together = __popc(__ballot_sync(kFull, how == kMid)) >= 8;
   if (how == kLane || (together && how == kMid)) {
-    x = lane_block_step<W>(g, bv, dv, bt, dt, (int32_t)t, u, A);
+    x = lane_block_step<W>(g, bv, dv, bt, dt, t, u, A);
     how = kDone;
   }
   __syncwarp();
@@ -809,19 +829,11 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
   while (wm) {
     const int src = __ffs(wm) - 1;
     wm &= wm - 1;
+    // (a shuffle from one lane: the compiler knows these to be the same in every lane and keeps
+    // them in uniform registers; through shared memory they cost the step 130 bytes of spills)
     const int64_t bv_ = __shfl_sync(kFull, bv, src), bt_ = __shfl_sync(kFull, bt, src);
-    BlockStep<W> st{g,
-                    A,
-                    bv_,
-                    bt_,
-                    __shfl_sync(kFull, dv, src),
-                    __shfl_sync(kFull, dt, src),
-                    __shfl_sync(kFull, (int32_t)t, src),
-                    lane,
-                    rec,
-                    cap,
-                    g.col + bv_,
-                    g.col + bt_};
+    BlockStep<W> st{g, A, bv_, bt_, __shfl_sync(kFull, dv, src), __shfl_sync(kFull, dt, src),
+                    __shfl_sync(kFull, t, src), lane, rec, cap, g.col + bv_, g.col + bt_};
 #ifdef N2V_STATS
     const long long t_enter = clock64();
 #endif

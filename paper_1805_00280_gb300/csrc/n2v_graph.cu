@@ -89,6 +89,7 @@ __global__ void k_validate_stats(const int64_t* __restrict__ rp, const int32_t* 
         break;
       }
       prev = x;
+      if (x == u) atomicOr(&sc[kScLoops], 1ull);
       if (w) {
         sum += w[j];
         wpre[j] = sum;
@@ -494,6 +495,7 @@ int n2v_graph_load(const int64_t* row_ptr, const int32_t* col, const uint32_t* w
     g->info.weighted = weighted;
     g->info.max_degree = (int64_t)sc[kScMaxDeg];
     g->info.max_wsum = (uint64_t)sc[kScMaxWsum];
+    g->view.loops = sc[kScLoops] != 0;
     g->info.w_min = weighted && nnz > 0 ? 0xffffffffu - (uint32_t)sc[kScWMin] : 1u;
     g->info.w_max = weighted && nnz > 0 ? (uint32_t)sc[kScWMax] : 1u;
     for (int i = 0; i < 34; ++i) g->info.deg_hist[i] = (int64_t)sc[kScHist + i];

@@ -88,6 +88,7 @@ struct GraphView {
   const int32_t* __restrict__ samples;
   const int32_t* __restrict__ tail;
   int64_t cut_block;
+  int loops;                             // some vertex is its own neighbour
 };
 
 // One walk job slice, as every sampler sees it.
@@ -98,6 +99,8 @@ struct WalkJob {
   int64_t count;       // walks in this slice
   int32_t l;
   uint32_t a_p, a_q;
+  uint64_t inv_q;      // floor((2^64 - 1) / a_q)
+  uint64_t inv_n;      // floor((2^64 - 1) / n_starts)
   uint64_t seed;
   int32_t* walks;      // [count][l]
   uint32_t* status;
@@ -107,6 +110,14 @@ struct WalkJob {
   int64_t approx_popular;  // popular: degree >= this
   uint32_t w_min, w_max;   // extreme edge weights of the graph
 };
+
+// floor(x / d) by the reciprocal inv = floor((2^64 - 1) / d): the estimate is the
+// quotient or one less.
+__device__ __forceinline__ uint64_t div_by(uint64_t x, uint64_t d, uint64_t inv) {
+  uint64_t q = __umul64hi(x, inv);
+  if (x - q * d >= d) ++q;
+  return q;
+}
 
 // Threads per block of the persistent kernels (the sampler and the serving tick).
 constexpr int kPersistThreads = 128;
@@ -411,6 +422,7 @@ enum : int {
   kScWMax = 43,
   kScSumDeg2 = 44,  // sum over edges of deg(target): entries of a stored transition table
   kScBmCount = 45,  // bitmap hubs assigned
+  kScLoops = 46,    // self-loops: not zero when there is one
   kScWords = 64
 };
 

@@ -29,15 +29,19 @@ struct DevSlice {
   int64_t count;
   int64_t slot_begin;   // prefix in the tick's slot space
   uint64_t seed;
+  uint64_t inv_q;       // floor((2^64 - 1) / a_q)
   int32_t l;
   uint32_t a_p, a_q;
   uint32_t pad;
 };
 
-// 96 registers a thread: five resident 128-thread blocks per SM (the default
-// grid).  KIND: the full or a lean instance (PersistKind).
+// Resident 128-thread blocks per SM: five at 96 registers a thread (the default
+// grid), eight at 64 through sampled blocks.
+constexpr int serve_per_sm(int kind) { return kind >= kPersistBlocks ? 8 : 5; }
+
+// KIND: the full instance, a lean one or one through sampled blocks (PersistKind).
 template <int KIND>
-__global__ void __launch_bounds__(kPersistThreads, 5)
+__global__ void __launch_bounds__(kPersistThreads, serve_per_sm(KIND))
     k_serve(GraphView g, const DevSlice* __restrict__ slices, int nslices, int64_t total_slots,
             unsigned long long* __restrict__ counter, LaunchCfg L, uint32_t* __restrict__ spill, uint32_t* status) {
   constexpr bool BLOCKS = KIND == kPersistBlocks || KIND == kPersistBlocksUnw;
@@ -77,7 +81,7 @@ __global__ void __launch_bounds__(kPersistThreads, 5)
       int64_t t = -1, v = -1;
       bool alive = false;
       if (mine) {
-        const int64_t s0 = S.starts[wid % S.n_starts];
+        const int64_t s0 = S.starts[wid];  // (one walk from each start: wid < n_starts)
         if (s0 >= 0 && s0 < g.n) {
           v = s0;
           alive = true;
@@ -85,7 +89,7 @@ __global__ void __launch_bounds__(kPersistThreads, 5)
           atomicOr(status, kStInvalidArg);
         }
       }
-      const StepArgs A{S.a_p, S.a_q, ~0ull / (uint64_t)S.a_q, S.seed};
+      const StepArgs A{S.a_p, S.a_q, S.inv_q, S.seed};
       int k = 0;
       for (; k < S.l; ++k) {
         if (sm.timed_out || !__any_sync(kFull, alive)) break;
@@ -96,7 +100,7 @@ __global__ void __launch_bounds__(kPersistThreads, 5)
         J.approx = 0;
         int32_t x;
         if (BLOCKS)
-          x = blocks_step<KIND == kPersistBlocks>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec,
+          x = blocks_step<KIND == kPersistBlocks, false>(g, alive, (int32_t)t, (int32_t)v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec,
                                                   block_records(L), lane);
         else
           x = warp_binned_step<KIND == kPersistFull>(g, alive, t, v, k, (uint64_t)wid, J, L.thread_max_deg, sm,
@@ -354,6 +358,7 @@ int n2v_serve_step(n2v_server* s, int* launched) {
     d.l = j.spec.l;
     d.a_p = j.a_p;
     d.a_q = j.a_q;
+    d.inv_q = ~0ull / j.a_q;
     s->host_slices.push_back(d);
     t.shares.push_back({id, take});
     j.launched += take;
@@ -377,6 +382,7 @@ int n2v_serve_step(n2v_server* s, int* launched) {
   const int kind = persist_kind(L, s->g->view, false);
   const bool blocks = kind == kPersistBlocks || kind == kPersistBlocksUnw;
   const int smem = (L.block_threads / 32) * (blocks ? block_smem_words(L) * 4 : warp_smem_bytes(L));
+  if (blocks && s->g->tune.blocks_per_sm <= 0) L.blocks = s->g->sms * serve_per_sm(kind);  // (no spill area to fit)
   auto kern = kind == kPersistBlocksUnw   ? k_serve<kPersistBlocksUnw>
               : kind == kPersistBlocks    ? k_serve<kPersistBlocks>
               : kind == kPersistLeanUnw ? k_serve<kPersistLeanUnw>

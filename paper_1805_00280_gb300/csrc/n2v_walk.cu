@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
 }
 
 // Persistent through sampled blocks: the same loop with blocks_step.
-template <int MINB, bool W>
+template <int MINB, bool W, bool APPROX>
 __global__ void __launch_bounds__(kPersistThreads, MINB)
     k_persistent_smp(GraphView g, WalkJob J, unsigned long long* __restrict__ counter, LaunchCfg L,
                       uint32_t* __restrict__) {
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t* rec = (uint32_t*)smem_raw + warp * block_smem_words(L);
-  const StepArgs A{J.a_p, J.a_q, ~0ull / (uint64_t)J.a_q, J.seed};
+  const StepArgs A{J.a_p, J.a_q, J.inv_q, J.seed};
 #ifdef N2V_STATS
   const long long t_kernel = clock64();
 #endif
@@ -179,10 +179,10 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
     const bool mine = lane < take && i < J.count;
     const int64_t wid = J.walk_begin + i;
     int32_t* row = J.walks + i * (int64_t)J.l;
-    int64_t t = -1, v = -1;
+    int32_t t = -1, v = -1;
     bool alive = false;
     if (mine) {
-      const int64_t s0 = J.starts[wid % J.n_starts];
+      const int32_t s0 = J.starts[(uint64_t)wid - div_by((uint64_t)wid, (uint64_t)J.n_starts, J.inv_n) * (uint64_t)J.n_starts];
       if (s0 >= 0 && s0 < g.n) {
         v = s0;
         alive = true;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
     for (; k < J.l; ++k) {
       if (!__any_sync(kFull, alive)) break;
       const int32_t x =
-          blocks_step<W>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec, block_records(L), lane);
+          blocks_step<W, APPROX>(g, alive, t, v, k, (uint64_t)wid, J, A, L.thread_max_deg, rec, block_records(L), lane);
       N2V_CHECK(g, !alive || (x >= -1 && x < g.n));
       if (mine) row[k] = alive ? x : -1;
       if (alive) {
@@ -339,7 +339,7 @@ static int smem_per_block(const LaunchCfg& c) {
 // latency.
 static int persistent_minb(int per_sm) { return per_sm <= 4 ? 4 : per_sm <= 5 ? 5 : per_sm <= 6 ? 6 : 8; }
 
-static const void* persistent_fn(int minb, bool blk, int kind) {
+static const void* persistent_fn(int minb, bool blk, int kind, bool approx) {
   if (blk) {
     switch (minb) {
       case 4: return (const void*)k_persistent_blk<4>;
@@ -349,19 +349,21 @@ static const void* persistent_fn(int minb, bool blk, int kind) {
     }
   }
   if (kind == kPersistBlocksUnw) {
+    if (approx) return (const void*)k_persistent_smp<5, false, true>;
     switch (minb) {
-      case 4: return (const void*)k_persistent_smp<4, false>;
-      case 6: return (const void*)k_persistent_smp<6, false>;
-      case 8: return (const void*)k_persistent_smp<8, false>;
-      default: return (const void*)k_persistent_smp<5, false>;
+      case 4: return (const void*)k_persistent_smp<4, false, false>;
+      case 6: return (const void*)k_persistent_smp<6, false, false>;
+      case 8: return (const void*)k_persistent_smp<8, false, false>;
+      default: return (const void*)k_persistent_smp<5, false, false>;
     }
   }
   if (kind == kPersistBlocks) {
+    if (approx) return (const void*)k_persistent_smp<5, true, true>;
     switch (minb) {
-      case 4: return (const void*)k_persistent_smp<4, true>;
-      case 6: return (const void*)k_persistent_smp<6, true>;
-      case 8: return (const void*)k_persistent_smp<8, true>;
-      default: return (const void*)k_persistent_smp<5, true>;
+      case 4: return (const void*)k_persistent_smp<4, true, false>;
+      case 6: return (const void*)k_persistent_smp<6, true, false>;
+      case 8: return (const void*)k_persistent_smp<8, true, false>;
+      default: return (const void*)k_persistent_smp<5, true, false>;
     }
   }
   if (kind == kPersistLeanUnw) {
@@ -394,23 +396,30 @@ static int launch_kind(const LaunchCfg& L, const GraphView& g, const WalkJob& J)
   return L.block_min_deg > 0 ? kPersistFull : persist_kind(L, g, J.approx != 0);
 }
 // Resident 128-thread blocks per SM of the sampled-block instances when the tuning
-// names none.
-constexpr int kBlockStepPerSm = 6;
+// names none: 64 registers a thread.  Steps on lanes (short lists) take 80: a round of
+// their warps is long enough as it is.  Measured with 8 / 6 / 5: R-MAT 24 117 / 131 / 143
+// ms, WeC-20 37 / 41 / 44 ms, ER 1.93 / 1.65 / 2.02 ms.  A job of no more walkers than
+// warps is as long as one walk, and takes 96 (999 walks: 0.67 / 0.60 / 0.56 ms).
+constexpr int kBlockStepPerSm = 8, kLaneStepPerSm = 6, kFewStepPerSm = 5;
 
 // The sampled-block instances use no spill area and a quarter of the shared memory,
-// so their grid is their own: the tuning's resident warps per SM, or 24.
+// so their grid is their own.
 static void block_step_grid(const n2v_graph* g, const WalkJob& J, LaunchCfg& L) {
   const int warps = g->tune.blocks_per_sm * (g->tune.block_threads / 32);
-  int per_sm = warps > 0 ? (warps + 3) / 4 : kBlockStepPerSm;
+  L.lane_walks = J.a_q == kAlphaOne || lane_walks(g->info);
+  const bool few = J.count <= (int64_t)g->sms * kFewStepPerSm * (kPersistThreads / 32);
+  int per_sm = warps > 0      ? (warps + 3) / 4
+               : few          ? kFewStepPerSm
+               : L.lane_walks ? kLaneStepPerSm
+                              : kBlockStepPerSm;
   const int smem = (L.block_threads / 32) * block_smem_words(L) * 4;
   per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
   L.minb = persistent_minb(per_sm);
   L.blocks = g->sms * std::min(per_sm, 8);
-  L.lane_walks = J.a_q == kAlphaOne || lane_walks(g->info);
 }
 
 static const void* persistent_fn(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
-  return persistent_fn(L.minb, L.block_min_deg > 0, launch_kind(L, g, J));
+  return persistent_fn(L.minb, L.block_min_deg > 0, launch_kind(L, g, J), J.approx != 0);
 }
 // Its dynamic shared memory.
 static int persistent_smem(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {
@@ -490,7 +499,7 @@ LaunchCfg resolve_launch(const n2v_graph* g, int variant) {
     const int warps = g->tune.blocks_per_sm > 0 ? g->tune.blocks_per_sm * (g->tune.block_threads / 32) : 20;
     int per_sm = std::max(1, (warps + 3) / 4);
     const int smem = smem_per_block(c);
-    const void* fn = persistent_fn(8, c.block_min_deg > 0, kPersistFull);  // the fewest registers: only shared memory limits it
+    const void* fn = persistent_fn(8, c.block_min_deg > 0, kPersistFull, false);  // the fewest registers: only shared memory limits it
     if (smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     int occ = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, c.block_threads, smem) == cudaSuccess && occ > 0)
@@ -546,6 +555,8 @@ static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) 
   J.l = c.l;
   J.a_p = c.a_p;
   J.a_q = c.a_q;
+  J.inv_q = ~0ull / c.a_q;
+  J.inv_n = ~0ull / (uint64_t)c.n_starts;
   J.seed = c.seed;
   J.walks = c.walks;
   J.status = g->status;
@@ -955,6 +966,8 @@ extern "C" int n2v_walk_noalloc(const n2v_graph* g, const int32_t* starts, int64
   J.l = l;
   J.a_p = a_p;
   J.a_q = a_q;
+  J.inv_q = ~0ull / a_q;
+  J.inv_n = ~0ull / (uint64_t)n_starts;
   J.seed = seed;
   J.status = g->status;
   J.approx = 0;
