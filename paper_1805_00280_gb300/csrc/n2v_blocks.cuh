@@ -280,7 +280,7 @@ __host__ __device__ __forceinline__ int block_smem_words(const LaunchCfg& L) { r
 template <bool W>
 struct BlockStep {
   // Chunks of a batch.  With weights two: four are 4,200 instructions and 300 bytes of spills,
-  // and weighted R-MAT 23 takes 160 ms instead of 143 ms; without, two cost R-MAT 24 133 ms
+  // and weighted R-MAT 23 took 160 ms instead of 143 ms; without, two cost R-MAT 24 133 ms
   // instead of 117 ms.
   static constexpr int kB = W ? 2 : 4;
   using Sum = typename std::conditional<W, uint64_t, uint32_t>::type;  // of hits, or of their weights
@@ -408,7 +408,9 @@ struct BlockStep {
     int left, gi;          // of the current group: chunks to come, and its record
     int pt;                // index of the key equal to t that this lane saw, or -1
     int32_t nx[kB], ns[4];  // the next batch's keys and samples
-    Sum sum, before;       // hits so far, and before the group (with weights: this lane's share of their weights)
+    uint32_t w[kB];        // with weights: those of the last batch's hits (this lane's),
+    int owed;              // and its record
+    Sum sum;               // hits so far (with weights: this lane's share of their weights)
   };
 
   __device__ __forceinline__ void fetch(Pass& P, const BlockRow& r, int c) const {
@@ -431,11 +433,13 @@ struct BlockStep {
     }
   }
 
-  // One batch: chunks c .. c + kB - 1.
-  __device__ __forceinline__ void batch(Pass& P, const BlockRow& r, int c, bool vk) {
+  // One batch: chunks c .. c + kB - 1 (with weights, c at the end only settles the last one).
+  __device__ __forceinline__ void batch(Pass& P, const BlockRow& r, int c, int c1, bool vk) {
     int32_t* win = (int32_t*)(rec + 2 * cap);
     int32_t x[kB];
     int node[kB];
+    Block b[kB];
+    if (!W || c < c1) {
 #pragma unroll
     for (int e = 0; e < kB; ++e) x[e] = P.nx[e];
     // the batch's largest key
@@ -473,7 +477,6 @@ struct BlockStep {
       block_search<kB>(r, P.from, x, node);
       P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
     }
-    Block b[kB];
     if (r.cut < 0) {
 #pragma unroll
       for (int e = 0; e < kB; ++e) b[e] = block_at(r.blk + 8ll * node[e]);
@@ -482,6 +485,11 @@ struct BlockStep {
       for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
     }
     if (32 * (c + kB) < P.nk) fetch(P, r, c + kB);
+    }
+    if (W) {
+      settle(P);
+      if (c >= c1) return;
+    }
     bool has_t = false;
 #pragma unroll
     for (int e = 0; e < kB; ++e) has_t = has_t || x[e] == t;
@@ -491,27 +499,23 @@ struct BlockStep {
     }
     bool in[kB];
     match(r, P.keys, 32 * c, node, x, b, in);
+    const Sum before = P.sum;
     uint32_t word[kB];
 #pragma unroll
     for (int e = 0; e < kB; ++e) {
       word[e] = __ballot_sync(kFull, in[e]);
       if (!W) {
         P.sum += __popc(word[e]);
-      } else {
+      } else {  // (the weights are waited for in settle, behind the next batch's loads)
         const int at = vk ? 32 * (c + e) + lane : block_pos(r, node[e], b[e], x[e]);
-        const uint32_t wx = in[e] ? __ldg(g.w + bv + at) : 0u;
-        P.sum += wx;
-        if (P.group == 1) {  // this chunk's weights, in two halves that cannot overflow
-          const uint64_t cs = (uint64_t)__reduce_add_sync(kFull, wx & 0xffffu) +
-                              ((uint64_t)__reduce_add_sync(kFull, wx >> 16) << 16);
-          if (lane == 0) {
-            put_total(P.gi + e, (Sum)cs);
-            rec[4 * (P.gi + e) + 2] = word[e];
-            block_of(P.gi + e) = (uint32_t)node[e];
-          }
+        P.w[e] = in[e] ? __ldg(g.w + bv + at) : 0u;
+        if (P.group == 1 && lane == 0) {
+          rec[4 * (P.gi + e) + 2] = word[e];
+          block_of(P.gi + e) = (uint32_t)node[e];
         }
       }
     }
+    P.owed = P.gi;
     if (P.group == 1) {
       if (!W && lane == 0) {
         if (kB == 4) {
@@ -524,18 +528,37 @@ struct BlockStep {
         }
       }
       P.gi += kB;
-    } else {
-      if (P.left == P.group && lane == 0) block_of(P.gi) = (uint32_t)node[0];
+    } else {  // the batch adds to its group's record
+      if (lane == 0) {
+        if (P.left == P.group) {
+          block_of(P.gi) = (uint32_t)node[0];
+          put_total(P.gi, 0);
+        }
+        if (!W) rec[P.gi] += P.sum - before;
+      }
       P.left -= kB;
-      if (P.left <= 0 || 32 * (c + kB) >= P.nk) {
-        const Sum gs = W ? (Sum)warp_sum_u64(P.sum - P.before) : (Sum)(P.sum - P.before);
-        if (lane == 0) put_total(P.gi, gs);
-        P.before = P.sum;
+      if (P.left <= 0) {
         P.left = P.group;
         ++P.gi;
       }
     }
     __syncwarp();  // the staged samples are read before the next batch's are written
+  }
+
+  // With weights: add the last batch's to the sum and to its records (before the first batch,
+  // nothing, to a record that comes to be written).
+  __device__ __forceinline__ void settle(Pass& P) {
+#pragma unroll
+    for (int e = 0; e < kB; ++e) {
+      P.sum += P.w[e];
+      // the chunk's weights, in two halves that cannot overflow
+      Sum cs = (Sum)__reduce_add_sync(kFull, P.w[e] & 0xffffu) +
+               ((Sum)__reduce_add_sync(kFull, P.w[e] >> 16) << (W ? 16 : 0));
+      if (lane == 0) {
+        if (P.group == 1) put_total(P.owed + e, cs);
+        else put_total(P.owed, total_at(P.owed, 2) + cs);
+      }
+    }
   }
 
   // Look chunks [c0, c1) of the keys up in the longer list; the samples before `from`
@@ -555,11 +578,14 @@ struct BlockStep {
     P.left = group;
     P.gi = 0;
     P.sum = 0;
-    P.before = 0;
     P.pt = -1;
+    P.owed = 0;
+#pragma unroll
+    for (int e = 0; e < kB; ++e) P.w[e] = 0;
     fetch(P, r, c0);
 #pragma unroll 1
-    for (int c = c0; c < c1; c += kB) batch(P, r, c, vk);
+    for (int c = c0; c < c1 + (W ? kB : 0); c += kB) batch(P, r, c, c1, vk);
+    if (W) __syncwarp();
     *pt = P.pt;
     return P.sum;
   }
@@ -724,15 +750,20 @@ struct BlockStep {
   __device__ __forceinline__ int behind(int prev, bool hit, uint64_t D, int pos_t, uint64_t t_part, uint64_t r) const {
     if (hit && base_before(prev + 1) + D + (pos_t >= 0 && pos_t < prev ? t_part : 0ull) > r) return prev;
     // behind prev every weight is the default, but for t
-    const bool passed = pos_t >= 0 && pos_t <= prev;
+    bool passed = pos_t >= 0 && pos_t <= prev;
     if (passed) D += t_part;
-    int j = first_above(prev, r - D);
-    if (pos_t >= 0 && !passed && j >= pos_t) {  // t lies in (prev, j]: nothing before it is above r
+    for (;;) {
+      const int j = first_above(prev, r - D);
+      if (pos_t < 0 || passed || j < pos_t) {
+        N2V_CHECK(g, j > prev && j < dv);
+        return j;
+      }
+      // t lies in (prev, j], and nothing before it is above r
       if (base_before(pos_t + 1) + D + t_part > r) return pos_t;
-      j = first_above(pos_t, r - D - t_part);
+      D += t_part;
+      prev = pos_t;
+      passed = true;
     }
-    N2V_CHECK(g, j > prev && j < dv);
-    return j;
   }
 
   // First position behind prev whose a_q W exceeds x (the last one if none does).
