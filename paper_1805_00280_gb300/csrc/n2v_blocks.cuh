@@ -157,12 +157,37 @@ __device__ __forceinline__ int32_t first_order_step(const GraphView& g, int64_t 
 }
 
 // ---------------------------------------------------------------------------
-// One lane, one step (k >= 1), 1 <= deg v <= kLaneDeg: each neighbour of v is
-// looked up in N(t), four at a time, and the hits are kept as a bit mask.
-// Thirty-two walkers of a warp go side by side, so a step of 20 neighbours costs
-// a warp about 20 look-ups for 32 steps, where the warp-wide form below pays its
-// fixed cost once for each.
-constexpr int kLaneDeg = 64;
+// One lane, one step (k >= 1), 1 <= deg v <= kLaneDeg: N(v) and N(t) are merged four
+// entries against four, one aligned 16-byte load for each four, and the hits are kept
+// as a bit mask.  Thirty-two walkers of a warp go side by side, so a step of 20
+// neighbours costs a warp about a dozen rounds for 32 steps, where the warp-wide form
+// below pays its fixed cost once for each.  When N(t) is much the longer list, the
+// lane goes to the next four of it that can hold a neighbour of v by a search of the
+// samples.
+// Bound: L1, whose every 16 bytes here belong to another line.  Measured (ER, 8M steps
+// of 20 neighbours): 1.62 ms with one look-up of samples and block for each
+// neighbour (112 sectors a step, L1 91% busy), 0.89 ms merged.
+// A lane with a longer N(t) than it can merge keeps only the shortest N(v): up to 64
+// R-MAT 20 (4, .25) took 120 ms, up to 8 114 ms.
+constexpr int kLaneDeg = 64, kJumpDeg = 8;
+
+// The longest N(t) that is merged four by four; behind it the lane searches.
+__device__ __forceinline__ int lane_reach(int dv) { return 4 * dv + 16; }
+
+// Entries 4 k .. 4 k + 3 of the aligned quads that hold the row [b, b + d) (k = 0 holds
+// its first entry); none in the place of other rows' entries.
+__device__ __forceinline__ int4 lane_quad(const GraphView& g, int64_t b, int d, int k, int32_t none) {
+  const int64_t q = (b >> 2) + k;
+  // (the quad that the end of col cuts is in the copy of its block)
+  const int32_t* p = (q >> 1) == g.cut_block ? g.tail + 4 * (int)(q & 1) : g.col + 4 * q;
+  int4 x = __ldg((const int4*)p);
+  const unsigned at = (unsigned)(4 * k - (int)(b & 3));
+  if (at >= (unsigned)d) x.x = none;
+  if (at + 1 >= (unsigned)d) x.y = none;
+  if (at + 2 >= (unsigned)d) x.z = none;
+  if (at + 3 >= (unsigned)d) x.w = none;
+  return x;
+}
 
 template <bool W>
 __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t bv, int dv, int64_t bt, int dt,
@@ -171,37 +196,38 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
   const uint64_t d1 = (uint64_t)kAlphaOne - (uint64_t)A.a_q, d2 = (uint64_t)A.a_p - (uint64_t)A.a_q;
   uint64_t hits = 0;
   int pt = kLaneDeg;  // index of t in N(v)
-  if (dt > 0) {
-    const BlockRow rt = block_row(g, bt, dt);
-    for (int i0 = 0; i0 < dv; i0 += 4) {
-      int32_t x[4];
-      int node[4];
-      Block b[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) x[e] = __ldg(nv + min(i0 + e, dv - 1));
-      block_search<4>(rt, 0, x, node);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) b[e] = block_load(rt, node[e]);
-      uint32_t m = 0, check = 0;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (block_has(b[e], x[e])) m |= 1u << e;
-        if (node[e] == 0 || node[e] == rt.n1) check |= 1u << e;
-        if (x[e] == t) pt = min(pt, i0 + e);
-      }
-#pragma unroll 1
-      for (check &= m; check; check &= check - 1) {  // perhaps a neighbouring row's entry
-        const int e = __ffs(check) - 1;
-        const int32_t y = __ldg(nv + min(i0 + e, dv - 1));
-        const int p = lower_bound32(g.col + bt, dt, y);
-        if (p >= dt || __ldg(g.col + bt + p) != y) m &= ~(1u << e);
-      }
-      hits |= (uint64_t)m << i0;
+  const int vlast = (int)(((bv + dv - 1) >> 2) - (bv >> 2)), tlast = (int)(((bt + dt - 1) >> 2) - (bt >> 2));
+  const bool jump = dt > lane_reach(dv);
+  int vi = 0, ti = 0;
+  int4 X = lane_quad(g, bv, dv, 0, -1), Y = lane_quad(g, bt, dt, 0, -2);
+  for (;;) {
+    const int at = 4 * vi - (int)(bv & 3);  // position of X.x (below 0: another row's)
+    const unsigned m = (X.x == Y.x || X.x == Y.y || X.x == Y.z || X.x == Y.w ? 1u : 0u) |
+                       (X.y == Y.x || X.y == Y.y || X.y == Y.z || X.y == Y.w ? 2u : 0u) |
+                       (X.z == Y.x || X.z == Y.y || X.z == Y.z || X.z == Y.w ? 4u : 0u) |
+                       (X.w == Y.x || X.w == Y.y || X.w == Y.z || X.w == Y.w ? 8u : 0u);
+    hits |= at >= 0 ? (uint64_t)m << at : (uint64_t)(m >> -at);
+    if (X.x == t || X.y == t || X.z == t || X.w == t) pt = at + (X.x == t ? 0 : X.y == t ? 1 : X.z == t ? 2 : 3);
+    const int32_t vmax = max(max(X.x, X.y), max(X.z, X.w)), tmax = max(max(Y.x, Y.y), max(Y.z, Y.w));
+    const bool next_v = vmax <= tmax || ti == tlast;
+    if (next_v && vi == vlast) break;
+    int k = (next_v ? vi : ti) + 1;
+    if (jump && !next_v) {
+      // the first of v's four that Y does not reach, and the block that can hold it
+      const int32_t y[1] = {X.x > tmax ? X.x : X.y > tmax ? X.y : X.z > tmax ? X.z : X.w};
+      int node[1];
+      const BlockRow rt = block_row(g, bt, dt);
+      block_search<1>(rt, 0, y, node);
+      k = min(tlast, max(k, (int)(2 * ((bt >> 3) + node[0]) - (bt >> 2))));
     }
-    hits &= ~0ull >> (64 - dv);  // the last key, repeated past the end, sets no bit of its own
-  } else {
-    for (int i = 0; i < dv; ++i)
-      if (__ldg(nv + i) == t) pt = i;
+    const int4 Z = lane_quad(g, next_v ? bv : bt, next_v ? dv : dt, k, next_v ? -1 : -2);
+    if (next_v) {
+      X = Z;
+      vi = k;
+    } else {
+      Y = Z;
+      ti = k;
+    }
   }
   if (pt < kLaneDeg) hits &= ~(1ull << pt);  // t weighs 1/p whatever N(t) holds
   if (!W) {
@@ -833,13 +859,13 @@ __device__ __forceinline__ int32_t blocks_step(const GraphView& g, bool alive, i
       // a dead end
     } else if (fixed || A.a_q == kAlphaOne) {
       x = first_order_step<W>(g, bv, dv, fixed ? -1 : t, u, fixed ? kAlphaOne : A.a_p);
-    } else if (dv <= min(thr, kLaneDeg)) {
+    } else if (dv <= min(thr, kLaneDeg) && dt <= lane_reach(dv)) {
       how = kLane;
     } else {
-      how = thr > 0 && dv <= kLaneDeg ? kMid : kWarp;
+      how = thr > 0 && dv <= (dt <= lane_reach(dv) ? kLaneDeg : kJumpDeg) ? kMid : kWarp;
     }
   }
-  // steps of up to kLaneDeg neighbours stay on their lanes when enough lanes have one
+  // other steps of up to kLaneDeg neighbours stay on their lanes when enough lanes have one
   const bool together = __popc(__ballot_sync(kFull, how == kMid)) >= 8;
   if (how == kLane || (together && how == kMid)) {
     x = lane_block_step<W>(g, bv, dv, bt, dt, t, u, A);
