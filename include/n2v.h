@@ -92,7 +92,7 @@ typedef struct n2v_tune {
                               and 64 registers a thread; the resident warps per SM (<= 16, 20,
                               24, more) select the budget.  Launches that step through sampled
                               blocks (graphs with samples, no hub cache, merge form or block
-                              tier) choose 32, 24 or 20 warps themselves where this is 0.     */
+                              tier) choose 20 to 32 warps themselves where this is 0.         */
   int32_t thread_max_deg;  /* a step runs on one lane when deg(v) and deg(t) are <= this      */
   int32_t smem_specials;   /* per-warp shared-memory slots for the special positions of a step */
   int32_t hub_count;       /* vertices (largest degree first) with a hashed neighbour set     */
@@ -154,7 +154,7 @@ typedef struct n2v_graph_info {
  * counterparts of the FN-Cache neighbour cache, Section 3.4): hashed
  * neighbour sets (8 bytes per slot) and rank bitmaps (16 bytes per 64
  * vertices of the graph, per bitmap hub), and last the samples of col: one
- * entry of every eight, half a byte for each entry.  n2v_graph_load also takes
+ * entry of every eight and of every 64, 9/16 of a byte for each entry.  n2v_graph_load also takes
  * an aux that lacks only the room for the samples; walks are slower then. */
 int n2v_graph_aux_bytes(int64_t n, int64_t nnz, int weighted, const n2v_tune* t, size_t* bytes);
 

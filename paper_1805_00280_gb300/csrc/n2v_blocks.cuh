@@ -31,7 +31,10 @@ namespace n2v {
 struct BlockRow {
   const int32_t* __restrict__ smp;  // smp[i]: first entry of block i + 1, i < n1
   const int32_t* __restrict__ blk;  // block i at blk + 8 i
+  const int32_t* __restrict__ top;  // every eighth sample: top[i], i < n2, the first entry of group i + 1
   int n1;    // samples inside the row (its blocks are 0 .. n1)
+  int n2;    // of them, first of a group of eight blocks (64 entries, aligned in col)
+  int up;    // group i starts at block 8 i - up
   int head;  // entries of block 0 before the row
   int len;
   int cut;                           // the block that reaches past the end of col, or -1
@@ -44,6 +47,9 @@ __device__ __forceinline__ BlockRow block_row(const GraphView& g, int64_t b, int
   r.smp = g.samples + f + 1;
   r.blk = g.col + 8 * f;
   r.n1 = (int)(((b + d - 1) >> 3) - f);
+  r.top = g.top + (f >> 3) + 1;
+  r.n2 = (int)(((f + r.n1) >> 3) - (f >> 3));
+  r.up = (int)(f & 7);
   r.head = (int)(b & 7);
   r.len = d;
   r.cut = f + r.n1 == g.cut_block ? r.n1 : -1;
@@ -86,19 +92,34 @@ __device__ __forceinline__ int block_lower_bound(const BlockRow& r, int i, const
   return lo + lower_bound32(row + lo, hi - lo, x);
 }
 
+// The block of x, given its group i (the number of top samples <= x): eight samples in
+// one load.
+__device__ __forceinline__ int block_in_group(const BlockRow& r, int i, int32_t x) {
+  const int i0 = 8 * i - r.up;  // the group's first block (before the row's, for i = 0)
+  const Block s = block_at(r.smp + (i0 - 1));
+  unsigned m = 0;
+#pragma unroll
+  for (int j = 1; j < 8; ++j) m |= s.s[j] <= x ? 1u << j : 0u;
+  // blocks 1 .. n1 only: samples of other rows do not count
+  if (i0 < 0) m &= 0xffffffffu << (1 - i0);
+  if (i0 + 7 > r.n1) m &= (2u << (r.n1 - i0)) - 1u;
+  return max(i0, 0) + __popc(m);
+}
+
 // Blocks of N keys of one lane: the number of samples in [from, n1) at or below
 // each, plus from (N searches side by side).
 template <int N>
-__device__ __forceinline__ void block_search(const BlockRow& r, int from, const int32_t (&x)[N], int (&node)[N]) {
+__device__ __forceinline__ void block_search(const int32_t* __restrict__ smp, int n1, int from, const int32_t (&x)[N],
+                                             int (&node)[N]) {
 #pragma unroll
   for (int e = 0; e < N; ++e) node[e] = from;
-  const int n = r.n1 - from;
+  const int n = n1 - from;
   if (n <= 0) return;
   for (int st = 1 << (31 - __clz(n)); st > 0; st >>= 1) {
 #pragma unroll
     for (int e = 0; e < N; ++e) {
       const int at = node[e] + st;
-      if (at <= r.n1 && __ldg(r.smp + at - 1) <= x[e]) node[e] = at;
+      if (at <= n1 && __ldg(smp + at - 1) <= x[e]) node[e] = at;
     }
   }
 }
@@ -217,7 +238,7 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
       const int32_t y[1] = {X.x > tmax ? X.x : X.y > tmax ? X.y : X.z > tmax ? X.z : X.w};
       int node[1];
       const BlockRow rt = block_row(g, bt, dt);
-      block_search<1>(rt, 0, y, node);
+      block_search<1>(rt.smp, rt.n1, 0, y, node);
       k = min(tlast, max(k, (int)(2 * ((bt >> 3) + node[0]) - (bt >> 2))));
     }
     const int4 Z = lane_quad(g, next_v ? bv : bt, next_v ? dv : dt, k, next_v ? -1 : -2);
@@ -428,8 +449,11 @@ struct BlockStep {
     const int32_t* __restrict__ keys;  // this lane's key of chunk 0
     int nk;
     int32_t kmax;          // the last key
-    int stage;             // samples staged for a batch at first: 64 or 128; 0: searched in global memory
-    int from;              // samples at or below every key still to come
+    const int32_t* __restrict__ smp;  // what is staged: the samples, or the top ones
+    int n;                 // of the row
+    bool far;              // the top ones
+    int stage;             // staged for a batch at first: 64 or 128; 0: searched in global memory
+    int from;              // of them, at or below every key still to come
     int group;             // chunks that share one record (1, or a multiple of four)
     int left, gi;          // of the current group: chunks to come, and its record
     int pt;                // index of the key equal to t that this lane saw, or -1
@@ -449,8 +473,8 @@ struct BlockStep {
 #pragma unroll
       for (int e = 0; e < kB; ++e) P.nx[e] = 32 * e < n - lane ? __ldg(k + 32 * e) : kNoKey;
     }
-    const int32_t* q = r.smp + P.from + lane;
-    const int m = r.n1 - P.from - lane;
+    const int32_t* q = P.smp + P.from + lane;
+    const int m = P.n - P.from - lane;
     P.ns[0] = 0 < m ? __ldg(q) : INT32_MAX;
     P.ns[1] = 32 < m ? __ldg(q + 32) : INT32_MAX;
     if (P.stage > 64) {
@@ -471,7 +495,7 @@ struct BlockStep {
     // the batch's largest key
     const int32_t last = P.nk - 32 * c >= 32 * kB ? __shfl_sync(kFull, x[kB - 1], 31) : P.kmax;
     int below = kWin;  // staged samples at or below the last key
-    if (P.stage) {
+    if (!W || P.stage) {
       win[lane] = P.ns[0];
       win[32 + lane] = P.ns[1];
       below = (P.ns[0] <= last ? 1 : 0) + (P.ns[1] <= last ? 1 : 0);
@@ -486,7 +510,7 @@ struct BlockStep {
 #pragma unroll 2
         for (int q = P.stage; q < kWin; q += 32) {
           const int i = P.from + q + lane;
-          const int32_t s = i < r.n1 ? __ldg(r.smp + i) : INT32_MAX;
+          const int32_t s = i < P.n ? __ldg(P.smp + i) : INT32_MAX;
           win[q + lane] = s;
           more += s <= last ? 1 : 0;
         }
@@ -500,8 +524,12 @@ struct BlockStep {
       for (int e = 0; e < kB; ++e) node[e] += P.from;
       P.from += below;
     } else {
-      block_search<kB>(r, P.from, x, node);
+      block_search<kB>(P.smp, P.n, P.from, x, node);
       P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
+    }
+    if (!W && P.far) {
+#pragma unroll
+      for (int e = 0; e < kB; ++e) node[e] = block_in_group(r, node[e], x[e]);
     }
     if (r.cut < 0) {
 #pragma unroll
@@ -598,8 +626,15 @@ struct BlockStep {
     P.kmax = __ldg((vk ? nv : nt) + P.nk - 1);
     // samples beside a batch of 128 keys: sixteen times the ratio of the lists
     const int beside = r.len >> 3, nb = (P.nk + 32 * kB - 1) / (32 * kB);
-    P.stage = beside <= 48 * nb ? 64 : beside <= 400 * nb ? 128 : 0;
-    P.from = from;
+    // Beyond the ratio 8 the top samples are staged, and a key's group of eight samples is one
+    // more load.  (R-MAT 24: 116.5 ms with the samples of every ratio, 111 ms.  With weights the
+    // 150 instructions cost more than they give, 125 and 138 ms: there the samples are searched
+    // in global memory beyond the ratio 25.)
+    P.far = !W && beside > 128 * nb;
+    P.smp = P.far ? r.top : r.smp;
+    P.n = P.far ? r.n2 : r.n1;
+    P.stage = beside <= 48 * nb || (P.far && beside <= 8 * 48 * nb) ? 64 : W && beside > 400 * nb ? 0 : 128;
+    P.from = P.far ? (from + r.up) >> 3 : from;
     P.group = group;
     P.left = group;
     P.gi = 0;

@@ -15,6 +15,10 @@ namespace n2v {
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// The samples of col fill whole groups of eight, and the copy of col's cut block follows.
+__host__ __device__ static inline int64_t samples_fill(int64_t nnz) { return (nnz + 63) >> 6 << 3; }
+__host__ __device__ static inline int64_t samples_end(int64_t nnz) { return samples_fill(nnz) + 8; }
+
 AuxLayout aux_layout(int64_t n, int64_t nnz, int weighted, const n2v_tune& t) {
   AuxLayout L{};
   size_t off = 0;
@@ -56,7 +60,7 @@ AuxLayout aux_layout(int64_t n, int64_t nnz, int weighted, const n2v_tune& t) {
   if (L.bm_cap > 0)
     off += align256(std::max<size_t>(16 * (size_t)L.bm_cap * (size_t)L.bm_words, 4 * ((size_t)n + 2)));
   L.samples = off;  // one entry of every eight in col
-  off += align256(sizeof(int32_t) * (size_t)(((nnz + 31) >> 5 << 2) + 8));
+  off += align256(sizeof(int32_t) * (size_t)samples_end(nnz)) + align256(sizeof(int32_t) * (size_t)((nnz + 63) >> 6));
   L.total = off;
   return L;
 }
@@ -293,17 +297,20 @@ static int build_bitmaps(n2v_graph* g, const AuxLayout& L, cudaStream_t s) {
   return N2V_OK;
 }
 
-// samples[i] = col[8 i]: the first entry of every 32-byte block of col.
-// Behind them goes a copy of the block that the end of col cuts, so that every block
-// can be loaded whole.
+// samples[i] = col[8 i]: the first entry of every 32-byte block of col; the last group
+// of eight is filled up.  Behind them goes a copy of the block that the end of col
+// cuts, so that every block can be loaded whole, and top[i] = samples[8 i].
 __global__ void __launch_bounds__(256) k_samples(const int32_t* __restrict__ col, int64_t nnz,
-                                                 int32_t* __restrict__ samples) {
-  const int64_t blocks = (nnz + 7) >> 3;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < blocks; i += (int64_t)gridDim.x * blockDim.x)
-    samples[i] = __ldg(col + 8 * i);
+                                                 int32_t* __restrict__ samples, int32_t* __restrict__ top) {
+  const int64_t blocks = (nnz + 7) >> 3, fill = samples_fill(nnz);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < fill; i += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t x = i < blocks ? __ldg(col + 8 * i) : INT32_MAX;
+    samples[i] = x;
+    if ((i & 7) == 0) top[i >> 3] = x;
+  }
   if (blockIdx.x == 0 && threadIdx.x < 8) {
     const int64_t e = (nnz & ~7ll) + threadIdx.x;
-    samples[((nnz + 31) >> 5 << 2) + threadIdx.x] = e < nnz ? __ldg(col + e) : -1;
+    samples[fill + threadIdx.x] = e < nnz ? __ldg(col + e) : -1;
   }
 }
 
@@ -313,10 +320,12 @@ static int build_samples(n2v_graph* g, const AuxLayout& L, cudaStream_t s) {
   g->view.samples = nullptr;
   if (g->nnz == 0 || g->aux_bytes < L.total) return N2V_OK;
   int32_t* out = (int32_t*)((char*)g->aux + L.samples);
-  k_samples<<<g->sms * 8, 256, 0, s>>>(g->view.col, g->nnz, out);
+  int32_t* top = (int32_t*)((char*)out + align256(sizeof(int32_t) * (size_t)samples_end(g->nnz)));
+  k_samples<<<g->sms * 8, 256, 0, s>>>(g->view.col, g->nnz, out, top);
   if (cudaGetLastError() != cudaSuccess) return N2V_ERR_CUDA;
   g->view.samples = out;
-  g->view.tail = out + ((g->nnz + 31) >> 5 << 2);
+  g->view.top = top;
+  g->view.tail = out + samples_fill(g->nnz);
   g->view.cut_block = g->nnz & 7 ? g->nnz >> 3 : -1;
   return N2V_OK;
 }

@@ -86,6 +86,7 @@ struct GraphView {
   // n2v_blocks.cuh: samples[i] = col[8 i], i < ceil(nnz / 8) (null = none), and a copy of the
   // block that the end of col cuts (cut_block, or -1)
   const int32_t* __restrict__ samples;
+  const int32_t* __restrict__ top;       // top[i] = samples[8 i]
   const int32_t* __restrict__ tail;
   int64_t cut_block;
   int loops;                             // some vertex is its own neighbour

@@ -36,8 +36,8 @@ struct DevSlice {
 };
 
 // Resident 128-thread blocks per SM: five at 96 registers a thread (the default
-// grid), eight at 64 through sampled blocks.
-constexpr int serve_per_sm(int kind) { return kind >= kPersistBlocks ? 8 : 5; }
+// grid), eight at 64 through sampled blocks, seven at 72 with weights.
+constexpr int serve_per_sm(int kind) { return kind == kPersistBlocksUnw ? 8 : kind == kPersistBlocks ? 7 : 5; }
 
 // KIND: the full instance, a lean one or one through sampled blocks (PersistKind).
 template <int KIND>

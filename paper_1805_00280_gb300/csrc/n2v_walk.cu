@@ -353,6 +353,7 @@ static const void* persistent_fn(int minb, bool blk, int kind, bool approx) {
     switch (minb) {
       case 4: return (const void*)k_persistent_smp<4, false, false>;
       case 6: return (const void*)k_persistent_smp<6, false, false>;
+      case 7: return (const void*)k_persistent_smp<7, false, false>;
       case 8: return (const void*)k_persistent_smp<8, false, false>;
       default: return (const void*)k_persistent_smp<5, false, false>;
     }
@@ -362,6 +363,7 @@ static const void* persistent_fn(int minb, bool blk, int kind, bool approx) {
     switch (minb) {
       case 4: return (const void*)k_persistent_smp<4, true, false>;
       case 6: return (const void*)k_persistent_smp<6, true, false>;
+      case 7: return (const void*)k_persistent_smp<7, true, false>;
       case 8: return (const void*)k_persistent_smp<8, true, false>;
       default: return (const void*)k_persistent_smp<5, true, false>;
     }
@@ -400,7 +402,8 @@ static int launch_kind(const LaunchCfg& L, const GraphView& g, const WalkJob& J)
 // their warps is long enough as it is.  Measured with 8 / 6 / 5: R-MAT 24 117 / 131 / 143
 // ms, WeC-20 37 / 41 / 44 ms, ER 1.93 / 1.65 / 2.02 ms.  A job of no more walkers than
 // warps is as long as one walk, and takes 96 (999 walks: 0.67 / 0.60 / 0.56 ms).
-constexpr int kBlockStepPerSm = 8, kLaneStepPerSm = 6, kFewStepPerSm = 5;
+// Weighted steps need 72 registers (weighted R-MAT 23: 124 ms with 7, 133 ms with 8).
+constexpr int kBlockStepPerSm = 8, kWeightedStepPerSm = 7, kLaneStepPerSm = 6, kFewStepPerSm = 5;
 
 // The sampled-block instances use no spill area and a quarter of the shared memory,
 // so their grid is their own.
@@ -411,10 +414,11 @@ static void block_step_grid(const n2v_graph* g, const WalkJob& J, LaunchCfg& L) 
   int per_sm = warps > 0      ? (warps + 3) / 4
                : few          ? kFewStepPerSm
                : L.lane_walks ? kLaneStepPerSm
+               : g->weighted  ? kWeightedStepPerSm
                               : kBlockStepPerSm;
   const int smem = (L.block_threads / 32) * block_smem_words(L) * 4;
   per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
-  L.minb = persistent_minb(per_sm);
+  L.minb = std::max(4, std::min(per_sm, 8));
   L.blocks = g->sms * std::min(per_sm, 8);
 }
 
