@@ -314,7 +314,7 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
 // instructions a kernel waits for none, at 3,300 a seventh of the time, at 4,600 it
 // takes twice as long (R-MAT 20).  A separate form for one batch in registers saved a
 // fifth of WeC-20's instructions and was slower for that reason.
-constexpr int kWin = 512;         // staged samples per warp
+constexpr int kWin = 128;         // staged samples per warp
 constexpr int32_t kNoKey = -2;    // in the place of a key past the end: below every vertex, equal to none
 
 // Shared memory of one warp: cap record words, cap more (the blocks of the first
@@ -395,10 +395,6 @@ struct BlockStep {
 #pragma unroll
     for (int e = 0; e < NE; ++e) p[e] = w0;
     if (n >= 32) {
-      if (n >= 128) {
-        if (n >= 256) level<256>(p, x);
-        level<128>(p, x);
-      }
       if (n >= 64) level<64>(p, x);
       level<32>(p, x);
     }
@@ -413,21 +409,19 @@ struct BlockStep {
     for (int e = 0; e < NE; ++e) count[e] = (int)((p[e] - w0) >> 2);
   }
 
-  // Compare keys and blocks; the lane's first key is keys[i0], the others 32 apart.  A match in
-  // the row's first or last block may be an entry of a neighbouring row: there the row's own
-  // entries are searched (rare, and one copy of it).
+  // Compare keys and blocks; the lane's first key is keys[i0], the others 32 apart.  With edges, a
+  // block may be the row's first or last one and a match there an entry of a neighbouring row:
+  // then the row's own entries are searched (rare, and one copy of it).
   template <int NE>
-  __device__ __forceinline__ void match(const BlockRow& r, const int32_t* __restrict__ keys, int i0,
+  __device__ __forceinline__ void match(const BlockRow& r, bool edges, const int32_t* __restrict__ keys, int i0,
                                         const int (&node)[NE], const int32_t (&x)[NE], const Block (&bl)[NE],
                                         bool (&in)[NE]) const {
-    unsigned m = 0, check = g.loops ? 15u : 0u;
 #pragma unroll
-    for (int e = 0; e < NE; ++e) {
-      in[e] = block_has(bl[e], x[e]);
-      m |= in[e] ? 1u << e : 0u;
-      if (node[e] == 0 || node[e] == r.n1) check |= 1u << e;
-    }
-    check &= m;
+    for (int e = 0; e < NE; ++e) in[e] = block_has(bl[e], x[e]);
+    if (!edges) return;
+    unsigned check = 0;
+#pragma unroll
+    for (int e = 0; e < NE; ++e) check |= in[e] && (node[e] == 0 || node[e] == r.n1 || g.loops) ? 1u << e : 0u;
     if (check) {
       const int32_t* __restrict__ row = r.blk + r.head;
       unsigned no = 0;
@@ -466,13 +460,8 @@ struct BlockStep {
   __device__ __forceinline__ void fetch(Pass& P, const BlockRow& r, int c) const {
     const int32_t* k = P.keys + 32 * c;
     const int n = P.nk - 32 * c;
-    if (n >= 32 * kB) {
 #pragma unroll
-      for (int e = 0; e < kB; ++e) P.nx[e] = __ldg(k + 32 * e);
-    } else {
-#pragma unroll
-      for (int e = 0; e < kB; ++e) P.nx[e] = 32 * e < n - lane ? __ldg(k + 32 * e) : kNoKey;
-    }
+    for (int e = 0; e < kB; ++e) P.nx[e] = 32 * e < n - lane ? __ldg(k + 32 * e) : kNoKey;
     const int32_t* q = P.smp + P.from + lane;
     const int m = P.n - P.from - lane;
     P.ns[0] = 0 < m ? __ldg(q) : INT32_MAX;
@@ -489,12 +478,13 @@ struct BlockStep {
     int32_t x[kB];
     int node[kB];
     Block b[kB];
+    bool edges = P.from == 0 || g.loops;  // a key may lie in the row's first or last block
     if (!W || c < c1) {
 #pragma unroll
     for (int e = 0; e < kB; ++e) x[e] = P.nx[e];
     // the batch's largest key
     const int32_t last = P.nk - 32 * c >= 32 * kB ? __shfl_sync(kFull, x[kB - 1], 31) : P.kmax;
-    int below = kWin;  // staged samples at or below the last key
+    int below = 0;  // staged samples at or below the last key
     if (!W || P.stage) {
       win[lane] = P.ns[0];
       win[32 + lane] = P.ns[1];
@@ -505,20 +495,9 @@ struct BlockStep {
         below += (P.ns[2] <= last ? 1 : 0) + (P.ns[3] <= last ? 1 : 0);
       }
       below = __reduce_add_sync(kFull, below);
-      if (below == P.stage) {
-        int more = 0;
-#pragma unroll 2
-        for (int q = P.stage; q < kWin; q += 32) {
-          const int i = P.from + q + lane;
-          const int32_t s = i < P.n ? __ldg(P.smp + i) : INT32_MAX;
-          win[q + lane] = s;
-          more += s <= last ? 1 : 0;
-        }
-        below += __reduce_add_sync(kFull, more);
-      }
       __syncwarp();
     }
-    if (below < kWin) {
+    if (below < P.stage) {
       search_staged(win, below, x, node);
 #pragma unroll
       for (int e = 0; e < kB; ++e) node[e] += P.from;
@@ -526,18 +505,15 @@ struct BlockStep {
     } else {
       block_search<kB>(P.smp, P.n, P.from, x, node);
       P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
+      edges = true;
     }
+    edges = edges || P.from == P.n;
     if (!W && P.far) {
 #pragma unroll
       for (int e = 0; e < kB; ++e) node[e] = block_in_group(r, node[e], x[e]);
     }
-    if (r.cut < 0) {
 #pragma unroll
-      for (int e = 0; e < kB; ++e) b[e] = block_at(r.blk + 8ll * node[e]);
-    } else {
-#pragma unroll
-      for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
-    }
+    for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
     if (32 * (c + kB) < P.nk) fetch(P, r, c + kB);
     }
     if (W) {
@@ -552,7 +528,7 @@ struct BlockStep {
       for (int e = 0; e < kB; ++e) P.pt = x[e] == t ? 32 * (c + e) + lane : P.pt;
     }
     bool in[kB];
-    match(r, P.keys, 32 * c, node, x, b, in);
+    match(r, edges, P.keys, 32 * c, node, x, b, in);
     const Sum before = P.sum;
     uint32_t word[kB];
 #pragma unroll
@@ -626,14 +602,15 @@ struct BlockStep {
     P.kmax = __ldg((vk ? nv : nt) + P.nk - 1);
     // samples beside a batch of 128 keys: sixteen times the ratio of the lists
     const int beside = r.len >> 3, nb = (P.nk + 32 * kB - 1) / (32 * kB);
-    // Beyond the ratio 8 the top samples are staged, and a key's group of eight samples is one
-    // more load.  (R-MAT 24: 116.5 ms with the samples of every ratio, 111 ms.  With weights the
+    // Beyond the ratio 4 the top samples are staged, and a key's group of eight samples is one
+    // more load; beyond 64 a batch's window outgrows the staging area and is searched in global
+    // memory.  (R-MAT 24: 116.5 ms with the samples of every ratio, 109 ms.  With weights the
     // 150 instructions cost more than they give, 125 and 138 ms: there the samples are searched
-    // in global memory beyond the ratio 25.)
-    P.far = !W && beside > 128 * nb;
+    // in global memory beyond the ratio 8.)
+    P.far = !W && beside > 64 * nb;
     P.smp = P.far ? r.top : r.smp;
     P.n = P.far ? r.n2 : r.n1;
-    P.stage = beside <= 48 * nb || (P.far && beside <= 8 * 48 * nb) ? 64 : W && beside > 400 * nb ? 0 : 128;
+    P.stage = beside <= 48 * nb || (P.far && beside <= 8 * 48 * nb) ? 64 : W && beside > 128 * nb ? 0 : 128;
     P.from = P.far ? (from + r.up) >> 3 : from;
     P.group = group;
     P.left = group;

@@ -349,7 +349,7 @@ static const void* persistent_fn(int minb, bool blk, int kind, bool approx) {
     }
   }
   if (kind == kPersistBlocksUnw) {
-    if (approx) return (const void*)k_persistent_smp<5, false, true>;
+    if (approx) return (const void*)k_persistent_smp<8, false, true>;
     switch (minb) {
       case 4: return (const void*)k_persistent_smp<4, false, false>;
       case 6: return (const void*)k_persistent_smp<6, false, false>;
@@ -359,7 +359,7 @@ static const void* persistent_fn(int minb, bool blk, int kind, bool approx) {
     }
   }
   if (kind == kPersistBlocks) {
-    if (approx) return (const void*)k_persistent_smp<5, true, true>;
+    if (approx) return (const void*)k_persistent_smp<7, true, true>;
     switch (minb) {
       case 4: return (const void*)k_persistent_smp<4, true, false>;
       case 6: return (const void*)k_persistent_smp<6, true, false>;
