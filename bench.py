@@ -105,7 +105,7 @@ def dist_env():
 # the sources the sampler kernels are compiled from (the autotuner, serving
 # loop, graph loader and the header's documentation are not part of them)
 KERNEL_SOURCES = ["paper_1805_00280_gb300/csrc/n2v_walk.cu", "paper_1805_00280_gb300/csrc/n2v_step.cuh",
-                  "paper_1805_00280_gb300/csrc/n2v_internal.cuh"]
+                  "paper_1805_00280_gb300/csrc/n2v_blocks.cuh", "paper_1805_00280_gb300/csrc/n2v_internal.cuh"]
 
 
 def csrc_digest() -> str:

@@ -92,7 +92,8 @@ typedef struct n2v_tune {
                               and 64 registers a thread; the resident warps per SM (<= 16, 20,
                               24, more) select the budget.  Launches that step through sampled
                               blocks (graphs with samples, no hub cache, merge form or block
-                              tier) choose 20 to 32 warps themselves where this is 0.         */
+                              tier) choose 20 to 32 warps themselves where this asks for the
+                              default 20.                                                     */
   int32_t thread_max_deg;  /* a step runs on one lane when deg(v) and deg(t) are <= this      */
   int32_t smem_specials;   /* per-warp shared-memory slots for the special positions of a step */
   int32_t hub_count;       /* vertices (largest degree first) with a hashed neighbour set     */

@@ -11,8 +11,8 @@
 // when they are not most blocks are never read.
 //
 // Measured (GB300, R-MAT 24, p = 2, q = 0.5): staging the whole longer list read
-// 55 KB of lists a step; the blocks read 24 KB from DRAM and run 262,144-walk
-// launches in 83 ms against 134 ms.  Hashed sets of every row (one 32-byte bucket
+// 55 KB of lists a step; the blocks read 26 KB from DRAM and run 262,144-walk
+// launches in 55 ms against 132 ms.  Hashed sets of every row (one 32-byte bucket
 // a key, an eighth of the instructions) were built and measured as well: DRAM gives
 // 64 bytes for each random 32, 71 KB a step, and the same launches took 155 ms.
 //
@@ -481,40 +481,40 @@ struct BlockStep {
     bool edges = P.from == 0 || g.loops;  // a key may lie in the row's first or last block
     if (!W || c < c1) {
 #pragma unroll
-    for (int e = 0; e < kB; ++e) x[e] = P.nx[e];
-    // the batch's largest key
-    const int32_t last = P.nk - 32 * c >= 32 * kB ? __shfl_sync(kFull, x[kB - 1], 31) : P.kmax;
-    int below = 0;  // staged samples at or below the last key
-    if (!W || P.stage) {
-      win[lane] = P.ns[0];
-      win[32 + lane] = P.ns[1];
-      below = (P.ns[0] <= last ? 1 : 0) + (P.ns[1] <= last ? 1 : 0);
-      if (P.stage > 64) {
-        win[64 + lane] = P.ns[2];
-        win[96 + lane] = P.ns[3];
-        below += (P.ns[2] <= last ? 1 : 0) + (P.ns[3] <= last ? 1 : 0);
+      for (int e = 0; e < kB; ++e) x[e] = P.nx[e];
+      // the batch's largest key
+      const int32_t last = P.nk - 32 * c >= 32 * kB ? __shfl_sync(kFull, x[kB - 1], 31) : P.kmax;
+      int below = 0;  // staged samples at or below the last key
+      if (!W || P.stage) {
+        win[lane] = P.ns[0];
+        win[32 + lane] = P.ns[1];
+        below = (P.ns[0] <= last ? 1 : 0) + (P.ns[1] <= last ? 1 : 0);
+        if (P.stage > 64) {
+          win[64 + lane] = P.ns[2];
+          win[96 + lane] = P.ns[3];
+          below += (P.ns[2] <= last ? 1 : 0) + (P.ns[3] <= last ? 1 : 0);
+        }
+        below = __reduce_add_sync(kFull, below);
+        __syncwarp();
       }
-      below = __reduce_add_sync(kFull, below);
-      __syncwarp();
-    }
-    if (below < P.stage) {
-      search_staged(win, below, x, node);
+      if (below < P.stage) {
+        search_staged(win, below, x, node);
 #pragma unroll
-      for (int e = 0; e < kB; ++e) node[e] += P.from;
-      P.from += below;
-    } else {
-      block_search<kB>(P.smp, P.n, P.from, x, node);
-      P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
-      edges = true;
-    }
-    edges = edges || P.from == P.n;
-    if (!W && P.far) {
+        for (int e = 0; e < kB; ++e) node[e] += P.from;
+        P.from += below;
+      } else {
+        block_search<kB>(P.smp, P.n, P.from, x, node);
+        P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
+        edges = true;
+      }
+      edges = edges || P.from == P.n;
+      if (!W && P.far) {
 #pragma unroll
-      for (int e = 0; e < kB; ++e) node[e] = block_in_group(r, node[e], x[e]);
-    }
+        for (int e = 0; e < kB; ++e) node[e] = block_in_group(r, node[e], x[e]);
+      }
 #pragma unroll
-    for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
-    if (32 * (c + kB) < P.nk) fetch(P, r, c + kB);
+      for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
+      if (32 * (c + kB) < P.nk) fetch(P, r, c + kB);
     }
     if (W) {
       settle(P);

@@ -29,7 +29,6 @@ struct DevSlice {
   int64_t count;
   int64_t slot_begin;   // prefix in the tick's slot space
   uint64_t seed;
-  uint64_t inv_q;       // floor((2^64 - 1) / a_q)
   int32_t l;
   uint32_t a_p, a_q;
   uint32_t pad;
@@ -89,7 +88,7 @@ __global__ void __launch_bounds__(kPersistThreads, serve_per_sm(KIND))
           atomicOr(status, kStInvalidArg);
         }
       }
-      const StepArgs A{S.a_p, S.a_q, S.inv_q, S.seed};
+      const StepArgs A{S.a_p, S.a_q, ~0ull / (uint64_t)S.a_q, S.seed};
       int k = 0;
       for (; k < S.l; ++k) {
         if (sm.timed_out || !__any_sync(kFull, alive)) break;
@@ -358,7 +357,6 @@ int n2v_serve_step(n2v_server* s, int* launched) {
     d.l = j.spec.l;
     d.a_p = j.a_p;
     d.a_q = j.a_q;
-    d.inv_q = ~0ull / j.a_q;
     s->host_slices.push_back(d);
     t.shares.push_back({id, take});
     j.launched += take;
@@ -382,7 +380,8 @@ int n2v_serve_step(n2v_server* s, int* launched) {
   const int kind = persist_kind(L, s->g->view, false);
   const bool blocks = kind == kPersistBlocks || kind == kPersistBlocksUnw;
   const int smem = (L.block_threads / 32) * (blocks ? block_smem_words(L) * 4 : warp_smem_bytes(L));
-  if (blocks && s->g->tune.blocks_per_sm <= 0) L.blocks = s->g->sms * serve_per_sm(kind);  // (no spill area to fit)
+  const int warps = s->g->tune.blocks_per_sm * (s->g->tune.block_threads / 32);
+  if (blocks && (warps <= 0 || warps == 20)) L.blocks = s->g->sms * serve_per_sm(kind);  // (no spill area to fit)
   auto kern = kind == kPersistBlocksUnw   ? k_serve<kPersistBlocksUnw>
               : kind == kPersistBlocks    ? k_serve<kPersistBlocks>
               : kind == kPersistLeanUnw ? k_serve<kPersistLeanUnw>

@@ -411,11 +411,12 @@ static void block_step_grid(const n2v_graph* g, const WalkJob& J, LaunchCfg& L) 
   const int warps = g->tune.blocks_per_sm * (g->tune.block_threads / 32);
   L.lane_walks = J.a_q == kAlphaOne || lane_walks(g->info);
   const bool few = J.count <= (int64_t)g->sms * kFewStepPerSm * (kPersistThreads / 32);
-  int per_sm = warps > 0      ? (warps + 3) / 4
-               : few          ? kFewStepPerSm
-               : L.lane_walks ? kLaneStepPerSm
-               : g->weighted  ? kWeightedStepPerSm
-                              : kBlockStepPerSm;
+  // (0 and 20 warps are the same request: the default, also as the autotuner writes it)
+  int per_sm = warps > 0 && warps != 20 ? (warps + 3) / 4
+               : few                    ? kFewStepPerSm
+               : L.lane_walks           ? kLaneStepPerSm
+               : g->weighted            ? kWeightedStepPerSm
+                                        : kBlockStepPerSm;
   const int smem = (L.block_threads / 32) * block_smem_words(L) * 4;
   per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
   L.minb = std::max(4, std::min(per_sm, 8));
