@@ -472,7 +472,9 @@ def run_ours(args):
                 "peak_kind": peak_kind,
                 "algorithmic_bytes_per_launch": [int(b) for b in abytes],
                 "kernel": {"persistent": "k_persistent", "binned": "k_binned_step", "plain": "k_plain_step"}[args.variant],
-                "bytes_model": "16 + 4 deg(v) (1+weighted) + [k>=1](16 + 4 deg(t)) + 4 per real transition"}
+                "bytes_model": "16 + 4 deg(v) (1+weighted) + [k>=1](16 + 4 deg(t)) + 4 per real transition",
+                "model_note": "counts both lists whole; the sampled blocks read only parts of the longer one, "
+                              "so frac is no bandwidth there and can pass 1"}
     # what the committed ncu capture's DRAM bytes come to over this run's call times
     roofline["dram"] = dram_fraction(dram, mean_launch_ms, peak)
     # the conservative lower model: N(v) and the output only, no N(t) message
