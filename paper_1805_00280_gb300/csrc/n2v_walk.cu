@@ -406,11 +406,12 @@ static int launch_kind(const LaunchCfg& L, const GraphView& g, const WalkJob& J)
 constexpr int kBlockStepPerSm = 8, kWeightedStepPerSm = 7, kLaneStepPerSm = 6, kFewStepPerSm = 5;
 
 // The sampled-block instances use no spill area and a quarter of the shared memory,
-// so their grid is their own.
-static void block_step_grid(const n2v_graph* g, const WalkJob& J, LaunchCfg& L) {
+// so their grid is their own.  J's parameters, and the walkers of one launch: a call in chunks
+// takes as many at a time.
+static void block_step_grid(const n2v_graph* g, const WalkJob& J, int64_t walkers, LaunchCfg& L) {
   const int warps = g->tune.blocks_per_sm * (g->tune.block_threads / 32);
   L.lane_walks = J.a_q == kAlphaOne || lane_walks(g->info);
-  const bool few = J.count <= (int64_t)g->sms * kFewStepPerSm * (kPersistThreads / 32);
+  const bool few = walkers <= (int64_t)g->sms * kFewStepPerSm * (kPersistThreads / 32);
   // (0 and 20 warps are the same request: the default, also as the autotuner writes it)
   int per_sm = warps > 0 && warps != 20 ? (warps + 3) / 4
                : few                    ? kFewStepPerSm
@@ -552,7 +553,7 @@ struct WalkCall {
 
 // Enqueue the launches of one call on stream s.
 static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) {
-  WalkJob J;
+  WalkJob J{};
   J.starts = c.starts;
   J.n_starts = c.n_starts;
   J.walk_begin = c.walk_begin;
@@ -588,15 +589,15 @@ static cudaError_t issue(const n2v_graph* g, const WalkCall& c, cudaStream_t s) 
     return cudaGetLastError();
   }
   // persistent
-  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, J, L);
+  const int64_t chunks = n_chunks(g, c.count);
+  const int64_t per = chunks == 1 ? c.count : g->tune.chunk_walkers;
+  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, J, per, L);
   const int psmem = persistent_smem(L, g->view, J);
   if (psmem > 48 * 1024)
     cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, psmem);
-  const int64_t chunks = n_chunks(g, c.count);
   unsigned long long* counters = (unsigned long long*)c.ws;
   cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * (size_t)chunks, s);
   if (e != cudaSuccess) return e;
-  const int64_t per = chunks == 1 ? c.count : g->tune.chunk_walkers;
   uint32_t* spill = L.spill_specials > 0 ? (uint32_t*)((char*)c.ws + counter_bytes(chunks)) : nullptr;
   for (int64_t ci = 0; ci < chunks; ++ci) {
     WalkJob Jc = J;
@@ -965,7 +966,7 @@ extern "C" int n2v_walk_noalloc(const n2v_graph* g, const int32_t* starts, int64
   // the scratch keeps the previous call's contents: the counters must start at 0
   if (cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * (size_t)chunks, s) != cudaSuccess)
     return N2V_ERR_CUDA;
-  WalkJob J;
+  WalkJob J{};
   J.starts = starts;
   J.n_starts = n_starts;
   J.l = l;
@@ -980,11 +981,11 @@ extern "C" int n2v_walk_noalloc(const n2v_graph* g, const int32_t* starts, int64
   J.approx_popular = 0;
   J.w_min = g->info.w_min;
   J.w_max = g->info.w_max;
-  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, J, L);
+  const int64_t per = chunks == 1 ? walk_count : g->tune.chunk_walkers;
+  if (launch_kind(L, g->view, J) >= kPersistBlocks) block_step_grid(g, J, per, L);
   const int smem = persistent_smem(L, g->view, J);
   if (smem > 48 * 1024)
     cudaFuncSetAttribute(persistent_fn(L, g->view, J), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  const int64_t per = chunks == 1 ? walk_count : g->tune.chunk_walkers;
   for (int64_t ci = 0; ci < chunks; ++ci) {
     const int64_t lo = ci * per;
     J.walk_begin = walk_begin + lo;
