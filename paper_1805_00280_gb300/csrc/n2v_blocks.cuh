@@ -21,6 +21,7 @@
 // only.
 #pragma once
 
+#include <algorithm>
 #include <type_traits>
 
 #include "n2v_step.cuh"
@@ -164,7 +165,7 @@ __device__ __forceinline__ int32_t first_order_step(const GraphView& g, int64_t 
   }
   const uint64_t m = r >> 16;  // first j with W_j > m
   if (!W) return __ldg(nv + m);
-  int lo = 0, n = dv;
+  int lo = 0, n = dv - 1;  // (the last position has W_j > m)
   while (n > 0) {
     const int half = n >> 1;
     if (__ldg(g.wpre + bv + lo + half) <= m) {
@@ -817,27 +818,36 @@ struct BlockStep {
 // Do most steps stay on their lanes?  Walks visit vertices about in proportion to
 // their degree, so the question is how many of the entries of col belong to rows
 // of at most kLaneDeg entries.
-inline bool lane_walks(const n2v_graph_info& info) {
+// Every first step does, and every step at q = 1 (blocks_step).
+inline bool lane_walks(const n2v_graph_info& info, int32_t l, uint32_t a_q) {
+  if (l == 1 || a_q == kAlphaOne) return true;
   int64_t small = 0;
   for (int i = 1; i < 34 && ((int64_t)1 << i) <= kLaneDeg; ++i) small += info.deg_hist[i] * (((int64_t)3 << i) / 4);
   return 2 * small > info.nnz;
 }
 
-// How many walkers a warp takes next, `seen` of `count` being taken.  Warp-wide
-// steps of one warp's walkers run one after another, so the fewer walkers a warp
-// has, the more warps share the job: half of what is left is spread evenly over
-// the warps, up to 32 each.  A small job then runs on as many warps as it has
-// walkers, and a large one ends on warps that finish together.  Where steps stay on
-// their lanes (L.lane_walks) 32 walkers cost a warp no more than one, and a job is
-// only spread so that one round of the warps takes it.
+// How many walkers a warp takes next of `count`, of which `counter` are taken, where the launch
+// does not say it (LaunchCfg::take).  Warp-wide steps of one warp's walkers run one after
+// another, so the fewer walkers a warp has, the more warps share the job: half of what is left
+// is spread evenly over the warps, up to 32 each.  A small job then runs on as many warps as it
+// has walkers, and a large one ends on warps that finish together.
 // Measured against 32 a warp throughout: 999 walks on R-MAT 20 7.5 -> 0.67 ms,
 // 524,288 on R-MAT 24 in two launches 167 -> 126 ms, 40 mixed serving jobs on R-MAT
 // 22 25.9 -> 9.0 ms.
-__device__ __forceinline__ int grab_size(const LaunchCfg& L, int64_t count, unsigned long long seen) {
+__device__ __forceinline__ int grab_size(int64_t count, const unsigned long long* counter) {
   const int64_t warps = (int64_t)gridDim.x * (kPersistThreads / 32);
-  const int64_t left = count - (int64_t)seen;
-  const int64_t even = L.lane_walks ? (count + warps - 1) / warps : left / (2 * warps);
-  return (int)max((int64_t)1, min((int64_t)32, even));
+  const int64_t left = count - (int64_t)*(const volatile unsigned long long*)counter;
+  return (int)max((int64_t)1, min((int64_t)32, left / (2 * warps)));
+}
+
+// Where steps stay on their lanes 32 walkers cost a warp no more than one, and the launch fixes the
+// walkers that a warp takes: a job is only spread so that one round of the warps takes it, and a
+// job of one short step a walker not at all.  Warps then do not read the counter, which costs the
+// others as much as their own turn at it.
+// Measured, one step from 131,072 vertices of R-MAT 20: 85 us by grab_size, 11 us; from 8,192 of a
+// path 14.7 us by an even spread with a look at the counter, 10.1 us without, 8.4 us by 32.
+inline int lane_take(int64_t walkers, int32_t l, int64_t warps) {
+  return l == 1 ? 32 : (int)std::min<int64_t>(32, (walkers + warps - 1) / warps);
 }
 
 // ---------------------------------------------------------------------------

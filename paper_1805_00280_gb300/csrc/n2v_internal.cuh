@@ -137,8 +137,7 @@ struct LaunchCfg {
   int block_min_deg;   // persistent sampler: 0 = warps independent; > 0 = block batches with a block tier
   int merge_ratio;     // x10, merge form of short steps (0: off)
   size_t l2_persist_bytes;  // bytes at the start of col marked persisting in L2 (0: off)
-  bool lane_walks;          // most steps stay on their lanes (grab_size)
-  int take;                 // serving: slots a warp takes at a time (0: grab_size)
+  int take;                 // walkers a warp takes at a time (0: grab_size)
 };
 
 // Instances of the persistent kernels.  kPersistBlocks steps through sampled

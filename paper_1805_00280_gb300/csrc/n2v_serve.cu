@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kPersistThreads, serve_per_sm(KIND))
     int take = L.take;
     unsigned long long base = 0;
     if (lane == 0) {
-      if (BLOCKS && take == 0) take = grab_size(L, total_slots, *(volatile unsigned long long*)counter);
+      if (BLOCKS && take == 0) take = grab_size(total_slots, counter);
       base = atomicAdd(counter, (unsigned long long)take);
     }
     base = __shfl_sync(kFull, base, 0);
@@ -310,9 +310,10 @@ static int32_t* job_rows(n2v_server* s, const Job& j) {
 // small jobs run on warps of their own.
 // Measured, a tick with grabs across the ends and with these: 512 jobs of one walk on R-MAT 16 with
 // a hub cache 17.6 and 1.67 ms; 200 jobs of 200 walks on ER 2.58 and 2.18 ms.
-static int tick_take(const std::vector<DevSlice>& shares, const LaunchCfg& L, bool blocks) {
+static int tick_take(const n2v_graph* g, const std::vector<DevSlice>& shares, const LaunchCfg& L, bool blocks) {
   if (!blocks) return 32;
-  if (!L.lane_walks) return 0;
+  for (const DevSlice& d : shares)
+    if (!lane_walks(g->info, d.l, d.a_q)) return 0;
   const int64_t warps = (int64_t)L.blocks * (L.block_threads / 32);
   for (int take = 1; take < 32; ++take) {
     int64_t grabs = 0;
@@ -386,12 +387,11 @@ int n2v_serve_step(n2v_server* s, int* launched) {
   }
   LaunchCfg L = resolve_launch(s->g, N2V_PERSISTENT);
   L.spill_specials = s->cfg.spill_specials;
-  L.lane_walks = lane_walks(s->g->info);
   const int kind = persist_kind(L, s->g->view, false);
   const bool blocks = kind == kPersistBlocks || kind == kPersistBlocksUnw;
   const int warps = s->g->tune.blocks_per_sm * (s->g->tune.block_threads / 32);
   if (blocks && (warps <= 0 || warps == 20)) L.blocks = s->g->sms * serve_per_sm(kind);  // (no spill area to fit)
-  L.take = tick_take(s->host_slices, L, blocks);
+  L.take = tick_take(s->g, s->host_slices, L, blocks);
   int64_t slots = 0;
   for (DevSlice& d : s->host_slices) {
     d.slot_begin = slots;

@@ -166,10 +166,10 @@ __global__ void __launch_bounds__(kPersistThreads, MINB)
   const long long t_kernel = clock64();
 #endif
   for (;;) {
-    int take = 32;
+    int take = L.take;
     unsigned long long base = 0;
     if (lane == 0) {
-      take = grab_size(L, J.count, *(volatile unsigned long long*)counter);
+      if (take == 0) take = grab_size(J.count, counter);
       base = atomicAdd(counter, (unsigned long long)take);
     }
     base = __shfl_sync(kFull, base, 0);
@@ -410,18 +410,19 @@ constexpr int kBlockStepPerSm = 8, kWeightedStepPerSm = 7, kLaneStepPerSm = 6, k
 // takes as many at a time.
 static void block_step_grid(const n2v_graph* g, const WalkJob& J, int64_t walkers, LaunchCfg& L) {
   const int warps = g->tune.blocks_per_sm * (g->tune.block_threads / 32);
-  L.lane_walks = J.a_q == kAlphaOne || lane_walks(g->info);
+  const bool lanes = lane_walks(g->info, J.l, J.a_q);
   const bool few = walkers <= (int64_t)g->sms * kFewStepPerSm * (kPersistThreads / 32);
   // (0 and 20 warps are the same request: the default, also as the autotuner writes it)
   int per_sm = warps > 0 && warps != 20 ? (warps + 3) / 4
                : few                    ? kFewStepPerSm
-               : L.lane_walks           ? kLaneStepPerSm
+               : lanes                  ? kLaneStepPerSm
                : g->weighted            ? kWeightedStepPerSm
                                         : kBlockStepPerSm;
   const int smem = (L.block_threads / 32) * block_smem_words(L) * 4;
   per_sm = std::max(1, std::min(per_sm, (227 << 10) / (smem + 1024)));
   L.minb = std::max(4, std::min(per_sm, 8));
   L.blocks = g->sms * std::min(per_sm, 8);
+  L.take = lanes ? lane_take(walkers, J.l, (int64_t)L.blocks * (kPersistThreads / 32)) : 0;
 }
 
 static const void* persistent_fn(const LaunchCfg& L, const GraphView& g, const WalkJob& J) {

@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from launches import captured
 from paper_1805_00280_gb300 import graphs as G
 from paper_1805_00280_gb300 import n2v
@@ -49,3 +50,16 @@ def test_the_grid_follows_the_walkers_of_one_launch(rmat14, weighted):
         assert launches(chunked, 16_000, noalloc=noalloc) == few * 160
     graph.close()
     chunked.close()
+
+
+@pytest.mark.parametrize("walks", [1, 33, 5000, 200_001])
+def test_jobs_of_one_step_stay_on_lanes(rmat14, walks):
+    """The first step does not read N(t): a job of one step is launched as a job at q = 1 is, whatever
+    the graph's degrees, and its rows are the oracle's."""
+    graph = n2v.Graph.from_csr(rmat14)
+    assert launches(graph, walks, l=1) == launches(graph, walks, l=1, q=1.0) == launches(graph, walks, q=1.0)
+    starts = np.arange(walks, dtype=np.int32) % rmat14.n
+    got = n2v.walk(graph, starts, 1, 1, 0.5, 2.0, 3).cpu().numpy()
+    want = oracle.walk(rmat14.row_ptr, rmat14.col, None, starts, 1, 0.5, 2.0, 3, np.arange(walks), threads=8)
+    np.testing.assert_array_equal(got, want)
+    graph.close()
