@@ -342,6 +342,9 @@ struct BlockStep {
   const int cap;
   const int32_t* __restrict__ nv;
   const int32_t* __restrict__ nt;
+#ifdef N2V_STATS
+  bool keys_v = false, searched = false;  // the keys are N(v); a batch was searched in global memory
+#endif
 
   __device__ __forceinline__ int records() const { return W ? cap >> 1 : cap; }
   // record i: total, ballot and first key's block
@@ -504,6 +507,9 @@ struct BlockStep {
         for (int e = 0; e < kB; ++e) node[e] += P.from;
         P.from += below;
       } else {
+#ifdef N2V_STATS
+        searched = true;
+#endif
         block_search<kB>(P.smp, P.n, P.from, x, node);
         P.from = __shfl_sync(kFull, node[kB - 1], 31);  // (of use only before a further batch)
         edges = true;
@@ -640,13 +646,11 @@ struct BlockStep {
   };
 
 #ifdef N2V_STATS
-  // As the generator modes of warp_step: keys searched in global memory (0, 1), or in staged
-  // samples (2, 3); keys N(v) are modes 0 and 3.
+  // As the generator modes of warp_step: steps with keys searched in global memory (0, 1), or in
+  // staged samples only (2, 3); keys N(v) are modes 0 and 3, and sh counts the keys.
   __device__ __forceinline__ void stat(long long t_enter) const {
-    const bool vk = dv <= max(dt, 128);
-    const int sh = vk ? dv : dt, lg = vk ? dt : dv;
-    const bool staged = (lg >> 3) <= 400 * ((sh + 127) >> 7);
-    const int m = staged ? (vk ? 3 : 2) : (vk ? 0 : 1);
+    const int sh = keys_v ? dv : dt, lg = keys_v ? dt : dv;
+    const int m = searched ? (keys_v ? 0 : 1) : (keys_v ? 3 : 2);
     if (lane == 0) {
       N2V_STAT(kStatMode + 4 * m, 1);
       N2V_STAT(kStatMode + 4 * m + 1, clock64() - t_enter);
@@ -664,6 +668,9 @@ struct BlockStep {
   __device__ __forceinline__ int run(uint64_t u) {
     // keys N(v) give positions without a search: also when they are the longer list but one batch
     const bool vk = dv <= max(dt, 32 * kB);
+#ifdef N2V_STATS
+    keys_v = vk;
+#endif
     const BlockRow row = vk ? block_row(g, bt, dt) : block_row(g, bv, dv);
     const Found f = search(u, vk, row);
     return f.chosen ? f.pos : behind(f.pos, f.hit, f.D, f.pos_t, f.t_part, f.r);
