@@ -65,8 +65,9 @@ extern "C" {
 #define N2V_ERR_CUDA (-6)          /* a CUDA runtime call failed                     */
 #define N2V_ERR_INTERNAL (-7)      /* a device self-check failed (checked build only: the
                                       library compiled with -DN2V_CHECKED verifies positions,
-                                      spill indices, search bounds and stored totals on the
-                                      device and records failures in the status word)   */
+                                      spill and record indices, search results and stored
+                                      totals on the device and records failures in the
+                                      status word)                                          */
 
 /* ---- sampler variants (n2v_walk `variant`) ------------------------------- */
 /* One thread per walker and one launch per step (the plain form). */

@@ -164,6 +164,7 @@ __device__ __forceinline__ int32_t first_order_step(const GraphView& g, int64_t 
     r -= jump;
   }
   const uint64_t m = r >> 16;  // first j with W_j > m
+  N2V_CHECK(g, m < (W ? __ldg(g.wpre + bv + dv - 1) : (uint64_t)dv));
   if (!W) return __ldg(nv + m);
   int lo = 0, n = dv - 1;  // (the last position has W_j > m)
   while (n > 0) {
@@ -242,6 +243,7 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
       block_search<1>(rt.smp, rt.n1, 0, y, node);
       k = min(tlast, max(k, (int)(2 * ((bt >> 3) + node[0]) - (bt >> 2))));
     }
+    N2V_CHECK(g, k > (next_v ? vi : ti) && k <= (next_v ? vlast : tlast));
     const int4 Z = lane_quad(g, next_v ? bv : bt, next_v ? dv : dt, k, next_v ? -1 : -2);
     if (next_v) {
       X = Z;
@@ -251,6 +253,8 @@ __device__ __forceinline__ int32_t lane_block_step(const GraphView& g, int64_t b
       ti = k;
     }
   }
+  N2V_CHECK(g, pt == kLaneDeg || (pt >= 0 && pt < dv && __ldg(nv + pt) == t));
+  N2V_CHECK(g, dv > 63 || (hits >> dv) == 0);
   if (pt < kLaneDeg) hits &= ~(1ull << pt);  // t weighs 1/p whatever N(t) holds
   if (!W) {
     const uint64_t T = (uint64_t)A.a_q * (uint64_t)dv + d1 * (uint64_t)__popcll(hits) + (pt < kLaneDeg ? d2 : 0ull);
@@ -413,6 +417,16 @@ struct BlockStep {
     for (int e = 0; e < NE; ++e) count[e] = (int)((p[e] - w0) >> 2);
   }
 
+#ifdef N2V_CHECKED
+  // i is the number of the n samples at or below x (a place past the end has no key).
+  __device__ void check_found(const int32_t* __restrict__ smp, int n, int i, int32_t x) const {
+    N2V_CHECK(g, i >= 0 && i <= n);
+    if (x == kNoKey || i < 0 || i > n) return;
+    N2V_CHECK(g, i == 0 || __ldg(smp + i - 1) <= x);
+    N2V_CHECK(g, i == n || __ldg(smp + i) > x);
+  }
+#endif
+
   // Compare keys and blocks; the lane's first key is keys[i0], the others 32 apart.  With edges, a
   // block may be the row's first or last one and a match there an entry of a neighbouring row:
   // then the row's own entries are searched (rare, and one copy of it).
@@ -501,6 +515,7 @@ struct BlockStep {
         below = __reduce_add_sync(kFull, below);
         __syncwarp();
       }
+      N2V_CHECK(g, below <= P.stage && P.stage <= kWin && P.from >= 0 && P.from + below <= P.n);
       if (below < P.stage) {
         search_staged(win, below, x, node);
 #pragma unroll
@@ -515,10 +530,16 @@ struct BlockStep {
         edges = true;
       }
       edges = edges || P.from == P.n;
+#ifdef N2V_CHECKED
+      for (int e = 0; e < kB; ++e) check_found(P.smp, P.n, node[e], x[e]);
+#endif
       if (!W && P.far) {
 #pragma unroll
         for (int e = 0; e < kB; ++e) node[e] = block_in_group(r, node[e], x[e]);
       }
+#ifdef N2V_CHECKED
+      for (int e = 0; e < kB; ++e) check_found(r.smp, r.n1, node[e], x[e]);
+#endif
 #pragma unroll
       for (int e = 0; e < kB; ++e) b[e] = block_load(r, node[e]);
       if (32 * (c + kB) < P.nk) fetch(P, r, c + kB);
@@ -545,6 +566,7 @@ struct BlockStep {
         P.sum += __popc(word[e]);
       } else {  // (the weights are waited for in settle, behind the next batch's loads)
         const int at = vk ? 32 * (c + e) + lane : block_pos(r, node[e], b[e], x[e]);
+        N2V_CHECK(g, !in[e] || (at >= 0 && at < dv && __ldg(nv + at) == x[e]));
         P.w[e] = in[e] ? __ldg(g.w + bv + at) : 0u;
         if (P.group == 1 && lane == 0) {
           rec[4 * (P.gi + e) + 2] = word[e];
@@ -553,6 +575,7 @@ struct BlockStep {
       }
     }
     P.owed = P.gi;
+    N2V_CHECK(g, P.gi >= 0 && P.gi + (P.group == 1 ? kB : 1) <= records());
     if (P.group == 1) {
       if (!W && lane == 0) {
         if (kB == 4) {
@@ -673,6 +696,7 @@ struct BlockStep {
 #endif
     const BlockRow row = vk ? block_row(g, bt, dt) : block_row(g, bv, dv);
     const Found f = search(u, vk, row);
+    N2V_CHECK(g, f.pos >= -1 && f.pos < dv);
     return f.chosen ? f.pos : behind(f.pos, f.hit, f.D, f.pos_t, f.t_part, f.r);
   }
 
@@ -767,6 +791,7 @@ struct BlockStep {
     bool live = p < dv;
     if (!vk) {
       if (hit) p = pos_of(plo, phi, __ldg(nt + p));
+      N2V_CHECK(g, !hit || (p >= plo && p < phi && __ldg(nv + p) == __ldg(nt + 32 * c + lane)));
       live = hit;
     }
     Sum incl, own = 1;
@@ -782,6 +807,7 @@ struct BlockStep {
                                        (pos_t >= 0 && pos_t < q ? t_part : 0ull) <= r;
     const unsigned m = __ballot_sync(kFull, below);
     const int f = 31 - __clz(m);
+    N2V_CHECK(g, c >= 0 && 32 * c < (vk ? dv : dt) && plo >= 0 && plo <= phi && phi <= dv);
     if (vk) return Found{min(32 * c + f + 1, dv - 1), true};
     int prev = plo - 1;
     if (m) {
