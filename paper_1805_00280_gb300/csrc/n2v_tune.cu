@@ -26,6 +26,26 @@ static const int kWarpTargets[] = {20, 16, 24};
 // (run-to-run spread on one sample is about 1%)
 static const float kMinGain = 0.02f;
 
+// Would launches under t step through sampled blocks (persist_kind)?  Hub caches come from vertices of
+// hub_min_degree and more.
+static bool by_blocks(const n2v_graph* g, const n2v_tune& t) {
+  const bool caches = (t.hub_count > 0 || t.bitmap_hubs > 0) &&
+                      g->info.max_degree >= std::max<int64_t>(1, t.hub_min_degree);
+  return g->view.samples && !caches && t.merge_ratio == 0 && t.block_min_deg == 0;
+}
+
+// Can cand and cur, which differ in one field, run at different speeds?  Steps through sampled blocks
+// stage nothing by bulk copies and have at most 256 records.  Their launches choose the warps by the
+// walkers they get (block_step_grid): a sample has fewer than the job, and what it favours (16 or 24
+// warps per SM) would hold back the job (R-MAT 24, 32 / 24 / 20 warps: 117 / 131 / 143 ms).  Measured
+// all the same, one of these fields came out changed on every small job tried, by the noise.
+static bool differs(const n2v_graph* g, const n2v_tune& cur, const n2v_tune& cand) {
+  if (!by_blocks(g, cur) || !by_blocks(g, cand)) return true;
+  return cand.stage_window == cur.stage_window && cand.stream_ratio == cur.stream_ratio &&
+         cand.stage_buffers == cur.stage_buffers && cand.blocks_per_sm == cur.blocks_per_sm &&
+         (cand.smem_specials == cur.smem_specials || std::min(cand.smem_specials, cur.smem_specials) < 256);
+}
+
 static size_t ws_for(const n2v_graph* g, int64_t sample, int32_t l, int warps_per_sm, int spill) {
   const int64_t chunks = g->tune.chunk_walkers > 0 ? (sample + g->tune.chunk_walkers - 1) / g->tune.chunk_walkers : 1;
   size_t b = ((sizeof(unsigned long long) * (size_t)chunks) + 255) & ~(size_t)255;
@@ -129,6 +149,7 @@ int n2v_autotune(n2v_graph* g, const int32_t* starts, int64_t n_starts, int32_t 
       if (cur.*(axes[a].field) == val) continue;
       n2v_tune cand = cur;
       cand.*(axes[a].field) = val;
+      if (!differs(g, cur, cand)) continue;
       // four windows of 1024 per warp do not fit beside 20 or more resident warps: skip that corner
       if (cand.stage_buffers * (cand.stage_window + 8) * 4 * (cand.block_threads / 32) * cand.blocks_per_sm > 200 * 1024)
         continue;
