@@ -204,9 +204,19 @@ def dram_fraction(dram_bytes_per_call, mean_call_ms: list, peak_gbs: float) -> d
     return {"achieved": gbs, "unit": "GB/s", "frac": gbs / peak_gbs}
 
 
+def sampler_kernel(variant: str, tune: dict, caches: int) -> str:
+    """The kernel that walks under this variant and tuning run, on a graph with its samples of col and
+    that many hub neighbour sets and bitmaps."""
+    if variant != "persistent":
+        return {"binned": "k_binned_step", "plain": "k_plain_step"}[variant]
+    if tune["block_min_deg"] > 0:
+        return "k_persistent_blk"
+    return "k_persistent" if caches or tune["merge_ratio"] else "k_persistent_smp"
+
+
 def effective_tune(tune: dict | None) -> dict | None:
-    """The tuning as the persistent sampler runs it: blocks_per_sm 0 means its default of 20
-    resident warps per SM, i.e. five 128-thread blocks."""
+    """The tuning as the persistent sampler runs it: blocks_per_sm 0 and 20 resident warps per SM,
+    i.e. five 128-thread blocks, are one request (the default)."""
     if tune is None:
         return None
     t = dict(tune)
@@ -471,7 +481,7 @@ def run_ours(args):
                 "traffic_source": f"profiles/traffic_{args.variant}_{wl.name}.json" if dram else None,
                 "peak_kind": peak_kind,
                 "algorithmic_bytes_per_launch": [int(b) for b in abytes],
-                "kernel": {"persistent": "k_persistent", "binned": "k_binned_step", "plain": "k_plain_step"}[args.variant],
+                "kernel": sampler_kernel(args.variant, tune.as_dict(), info.hub_count + info.bitmap_hubs),
                 "bytes_model": "16 + 4 deg(v) (1+weighted) + [k>=1](16 + 4 deg(t)) + 4 per real transition",
                 "model_note": "counts both lists whole; the sampled blocks read only parts of the longer one, "
                               "so frac is no bandwidth there and can pass 1"}
