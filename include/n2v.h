@@ -95,14 +95,21 @@ typedef struct n2v_tune {
                               blocks (graphs with samples, no hub cache, merge form or block
                               tier) choose 20 to 32 warps themselves where this asks for the
                               default 20.                                                     */
-  int32_t thread_max_deg;  /* a step runs on one lane when deg(v) and deg(t) are <= this      */
-  int32_t smem_specials;   /* per-warp shared-memory slots for the special positions of a step */
+  int32_t thread_max_deg;  /* a step runs on one lane when deg(v) and deg(t) are <= this.  Through
+                              sampled blocks: when deg(v) <= this (64 at most) and deg(t) <=
+                              4 deg(v) + 16; unless this is 0, other steps of up to 64 neighbours
+                              (8 where deg(t) is beyond that) too, where eight walkers of a warp
+                              have one; first steps and steps at q = 1 in any case              */
+  int32_t smem_specials;   /* per-warp shared-memory slots for the special positions of a step;
+                              through sampled blocks, records of 32 keys (at most 256 are used)  */
   int32_t hub_count;       /* vertices (largest degree first) with a hashed neighbour set     */
   int32_t hub_min_degree;  /* a vertex needs at least this degree to get a hashed set         */
   int32_t chunk_walkers;   /* walkers per persistent launch (0 = all in one launch)           */
   int32_t hub_budget_mb;   /* MiB of device memory for all hub hash sets (8 bytes per slot)   */
   int32_t stage_window;    /* elements per shared-memory window that stages the longer list of
-                              a step by TMA bulk copies (power of two, 64..4096; 0 = never) */
+                              a step by TMA bulk copies (power of two, 64..4096; 0 = never).
+                              This, stream_ratio, spill_specials and stage_buffers are not used
+                              by launches through sampled blocks                            */
   int32_t stream_ratio;    /* x10: stage the longer list when its length is at most
                               stream_ratio/10 * 32*ceil(short/32) * log2(long) (else probe it) */
   int32_t spill_specials;  /* per-warp device-workspace slots for special neighbours that do

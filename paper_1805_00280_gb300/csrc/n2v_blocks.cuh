@@ -1,7 +1,8 @@
 // The step through sampled blocks: membership in the longer list by a search of
 // its samples and one 32-byte block.
 //
-// col is read in blocks of eight entries (32 bytes: one DRAM sector), and the
+// col is read in blocks of eight entries (32 bytes: one DRAM sector where col lies on
+// 32 bytes, as an allocation does; on 16, which suffices, parts of two), and the
 // auxiliary buffer keeps the first entry of every block, samples[i] = col[8 i]
 // (built by n2v_graph_load; half a byte for each entry of col).  The block that
 // can hold x is found among a row's samples, an eighth of the row, and whether it
@@ -11,8 +12,8 @@
 // when they are not most blocks are never read.
 //
 // Measured (GB300, R-MAT 24, p = 2, q = 0.5): staging the whole longer list read
-// 55 KB of lists a step; the blocks read 26 KB from DRAM and run 262,144-walk
-// launches in 55 ms against 132 ms.  Hashed sets of every row (one 32-byte bucket
+// 55 KB of lists a step; the blocks move 28 KB of DRAM (5.65 TB/s) and run 262,144-walk
+// launches in 56 ms against 132 ms.  Hashed sets of every row (one 32-byte bucket
 // a key, an eighth of the instructions) were built and measured as well: DRAM gives
 // 64 bytes for each random 32, 71 KB a step, and the same launches took 155 ms.
 //
@@ -630,13 +631,15 @@ struct BlockStep {
     P.keys = (vk ? nv : nt) + lane;
     P.nk = vk ? dv : dt;
     P.kmax = __ldg((vk ? nv : nt) + P.nk - 1);
-    // samples beside a batch of 128 keys: sixteen times the ratio of the lists
+    // samples beside a batch: sixteen times the ratio of the lists (128 keys), with weights eight
+    // times (64 keys)
     const int beside = r.len >> 3, nb = (P.nk + 32 * kB - 1) / (32 * kB);
-    // Beyond the ratio 4 the top samples are staged, and a key's group of eight samples is one
-    // more load; beyond 64 a batch's window outgrows the staging area and is searched in global
-    // memory.  (R-MAT 24: 116.5 ms with the samples of every ratio, 109 ms.  With weights the
-    // 150 instructions cost more than they give, 125 and 138 ms: there the samples are searched
-    // in global memory beyond the ratio 8.)
+    // Without weights the top samples are staged beyond the ratio 4, and a key's group of eight
+    // samples is one more load; beyond 64 a batch's window outgrows the staging area and is
+    // searched in global memory.  (R-MAT 24: 116.5 ms with the samples themselves at every ratio,
+    // 111 ms so.)  With weights the 150 instructions of that cost more than they give (weighted
+    // R-MAT 23 138 ms against 125 ms): there the samples are staged up to the ratio 16 and searched
+    // in global memory beyond.
     P.far = !W && beside > 64 * nb;
     P.smp = P.far ? r.top : r.smp;
     P.n = P.far ? r.n2 : r.n1;

@@ -37,7 +37,7 @@ static bool by_blocks(const n2v_graph* g, const n2v_tune& t) {
 // Can cand and cur, which differ in one field, run at different speeds?  Steps through sampled blocks
 // stage nothing by bulk copies and have at most 256 records.  Their launches choose the warps by the
 // walkers they get (block_step_grid): a sample has fewer than the job, and what it favours (16 or 24
-// warps per SM) would hold back the job (R-MAT 24, 32 / 24 / 20 warps: 117 / 131 / 143 ms).  Measured
+// warps per SM) would hold back the job (R-MAT 24, 32 / 24 / 20 warps: 111 / 120 / 129 ms).  Measured
 // all the same, one of these fields came out changed on every small job tried, by the noise.
 static bool differs(const n2v_graph* g, const n2v_tune& cur, const n2v_tune& cand) {
   if (!by_blocks(g, cur) || !by_blocks(g, cand)) return true;

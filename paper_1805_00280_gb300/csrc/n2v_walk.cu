@@ -399,10 +399,11 @@ static int launch_kind(const LaunchCfg& L, const GraphView& g, const WalkJob& J)
 }
 // Resident 128-thread blocks per SM of the sampled-block instances when the tuning
 // names none: 64 registers a thread.  Steps on lanes (short lists) take 80: a round of
-// their warps is long enough as it is.  Measured with 8 / 6 / 5: R-MAT 24 117 / 131 / 143
-// ms, WeC-20 37 / 41 / 44 ms, ER 1.93 / 1.65 / 2.02 ms.  A job of no more walkers than
-// warps is as long as one walk, and takes 96 (999 walks: 0.67 / 0.60 / 0.56 ms).
-// Weighted steps need 72 registers (weighted R-MAT 23: 124 ms with 7, 133 ms with 8).
+// their warps is long enough as it is.  Measured with 8 / 6 / 5: R-MAT 24 111 / 120 / 129
+// ms, WeC-20 36.7 / 40.2 / 43.2 ms, ER 1.19 / 0.87 / 0.96 ms, R-MAT 20 at q = 1 1.56 / 1.17 /
+// 1.19 ms.  A job of no more walkers than warps is as long as one walk, and takes 96 (999
+// walks: 0.64 / 0.57 / 0.55 ms).  Weighted steps take 72: weighted R-MAT 23 121 / 122 / 134 ms
+// with 8 / 7 / 6.
 constexpr int kBlockStepPerSm = 8, kWeightedStepPerSm = 7, kLaneStepPerSm = 6, kFewStepPerSm = 5;
 
 // The sampled-block instances use no spill area and a quarter of the shared memory,
